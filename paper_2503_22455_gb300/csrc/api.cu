@@ -375,7 +375,7 @@ iim_status iim_problem_create(const iim_problem_desc* desc, const iim_options* o
   const bool iface = desc->bc == IIM_BC_INTERFACE;
   P.nfit_cap = iface ? 2 * P.K_cap : P.K_cap;
   IIM_ALLOC(P.fit_R, int32_t, P.nfit_cap);
-  IIM_ALLOC(P.fit_overflow, int, P.nfit_cap);
+  IIM_ALLOC(P.fit_later, int, P.nfit_cap + 1);
   IIM_ALLOC(P.fit_nodes, int32_t, (size_t)P.nfit_cap * P.rcap);
   IIM_ALLOC(P.fit_coef, double, (size_t)P.nfit_cap * (P.w + 1) * P.rcap);
   IIM_ALLOC(P.fit_cdat, double, (size_t)P.nfit_cap * (P.w + 1));
