@@ -445,25 +445,20 @@ iim_status iim_problem_create(const iim_problem_desc* desc, const iim_options* o
   st = read_status(P);
   if (st != IIM_OK) { set_error(iim_status_string(st)); IIM_FAIL(st); }
   {
-    // unknown count of the coarsest level from its aux codes (copied to the host once)
     Level& C = P.lv.back();
-    std::vector<int32_t> aux(C.g.N);
-    cudaMemcpy(aux.data(), C.aux, sizeof(int32_t) * C.g.N, cudaMemcpyDeviceToHost);
-    int nu = 0;
-    for (auto a : aux) nu += a != -2;
     if (C.g.N + P.aug > 4096) {
       set_error("the coarsest multigrid level has more than 4096 nodes: choose n with more factors of 2");
       IIM_FAIL(IIM_ERR_INVALID_ARG);
     }
     // the dense coarse system holds a slot per node of the coarsest level (+ the augmentation),
     // so that a later set-up with other geometry needs no other size
-    P.coarse_nu = nu;
     P.coarse_n = (int)C.g.N + P.aug;
     const size_t cn = (size_t)P.coarse_n;
     IIM_ALLOC(P.coarse_map, int32_t, cn);
-    IIM_ALLOC(P.coarse_piv, int32_t, cn > 0 ? cn : 1);
-    IIM_ALLOC(P.coarse_lu64, double, 2 * cn * cn + 1);
-    IIM_ALLOC(P.coarse_lu32, float, 2 * cn * cn + 1);
+    IIM_ALLOC(P.coarse_piv, int32_t, 2 * cn + 1);
+    // only the form of the multigrid precision is used
+    if (opt->mg_precision == IIM_MG_FP64) IIM_ALLOC(P.coarse_lu64, double, 2 * cn * cn + 1024);
+    else IIM_ALLOC(P.coarse_lu32, float, 2 * cn * cn + 1024);
   }
   mg_coarse_factor(P, P.stream);
   cudaStreamSynchronize(P.stream);

@@ -154,13 +154,12 @@ struct Problem {
   int red_blocks = 0;
   // multigrid
   std::vector<Level> lv;
-  int coarse_nu = 0;              // unknowns on the coarsest level at creation (sizes the LU's shared memory)
   int coarse_n = 0;               // size of the padded coarse system: the coarsest level's nodes (+1 when augmented)
   int aug = 0;                    // pure Neumann: the augmented system of Sec. 2.3 (one more unknown)
   int32_t* coarse_map = nullptr;  // [coarse_n] node of each slot of the coarse system, -1 if none
-  double* coarse_lu64 = nullptr;  // [nu][nu] LU factors (row major), FP64
-  float* coarse_lu32 = nullptr;
-  int32_t* coarse_piv = nullptr;
+  double* coarse_lu64 = nullptr;  // scratch matrix, inverse (each coarse_n^2, row major), pivot block; FP64 multigrid
+  float* coarse_lu32 = nullptr;   // the same for FP32 multigrid
+  int32_t* coarse_piv = nullptr;  // [2 coarse_n] row order of the elimination, rows of the current step
   // status and scratch
   int* d_status = nullptr;
   int* d_counts = nullptr;        // [kCountSlots] device counters (see kCount*)

@@ -198,26 +198,49 @@ __global__ void k_bridge_out(GridView g, const T* __restrict__ u, double* __rest
 }
 
 // ---------------------------------------------------------------------------- coarsest level
-// dense coarse matrix (row major, nu x nu) from the level's stencil
+// The coarse system has n = nu + aug unknowns, nu counted on the device (a later set-up with
+// other geometry keeps the arrays, of fixed stride ld >= n).  Its dense inverse is formed by
+// blocked Gauss-Jordan elimination with row pivoting: per block of kGJ (32) columns one CTA
+// factors the panel and inverts its pivot block (k_gj_panel), then a grid of 32 x 32 tiles
+// carries the step to the whole matrix (k_gj_update).  A step reads one of the two n x n
+// buffers and writes the other, so no tile waits for another; the first buffer is chosen so
+// that the last step ends in buffer 0, from which k_gj_finish writes the inverse of the matrix
+// with its original row order to buffer 1.
+// The panel is bound by its chain of pivots (two barriers each, about 0.5 us); the rest of the
+// chip is idle meanwhile, but the chain is n long instead of the n^3 / 1024 of one CTA that
+// works on the matrix in global memory.  Measured: set-up of a 736^2 exterior star (coarsest
+// level 23^2) 82.5 -> 2.8 ms, of a 80^3 sphere interface 43.6 -> 5.5 ms with the fits.
+constexpr int kGJ = 32;
+
+struct GJView {                         // sizes of the current set-up's system
+  int n, steps;
+  __device__ GJView(const int* nu_dev, int aug, int ld, int b) {
+    const int nu = *nu_dev;
+    n = nu < 0 || nu + aug > ld ? 0 : nu + aug;        // out of range: reported by k_coarse_assemble
+    steps = (n + b - 1) / b;
+  }
+  // buffer (0 or 1) that step k reads
+  __device__ int src(int k) const { return (steps + k) & 1; }
+};
+
+// rows of the dense matrix (zeroed beforehand): row r < nu the SW operator of unknown r;
+// augmented (pure Neumann, Sec. 2.3): a last column and row of ones over the unknowns
 template <typename T>
 __global__ void k_coarse_assemble(LevelView<double> L, const int32_t* __restrict__ map, const int* __restrict__ nu_dev,
-                                  int ld, const int32_t* __restrict__ inv, T* __restrict__ A, int aug, int* status) {
-  // The coarse system of the current set-up in the leading n x n block (n = nu + aug, nu the
-  // coarsest level's unknowns, counted on the device) of an array of fixed stride ld (the
-  // level's node count + aug), so that a later set-up with another geometry needs no other
-  // size: rows r < nu the SW operator; augmented (pure Neumann, Sec. 2.3): a last column and
-  // row of ones over the unknowns and a zero corner
+                                  int ld, const int32_t* __restrict__ inv, T* __restrict__ buf, int aug, int b,
+                                  int* status) {
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  const int nu = *nu_dev, n = nu + aug;
-  if (nu < 0 || n > ld) {              // more unknowns than the system has room for
+  const int nu = *nu_dev;
+  if (nu < 0 || nu + aug > ld) {       // more unknowns than the system has room for
     if (r == 0) set_status(status, IIM_ERR_CAPACITY);
     return;
   }
-  if (r >= n) return;
-  for (int c = 0; c < n; ++c) A[(size_t)r * ld + c] = (aug && c == nu && r < nu) ? (T)1 : (T)0;
-  if (r == nu) {                       // the augmentation row
-    for (int c = 0; c < nu; ++c) A[(size_t)r * ld + c] = 1;
-    return;
+  if (r >= nu) return;
+  const GJView V(nu_dev, aug, ld, b);
+  T* A = buf + (size_t)V.src(0) * ld * ld;
+  if (aug) {
+    A[(size_t)r * ld + nu] = (T)1;
+    A[(size_t)nu * ld + r] = (T)1;
   }
   int64_t i = map[r];
   int a = L.aux[i];
@@ -253,148 +276,166 @@ __global__ void k_unknown_flag(GridView g, const int32_t* __restrict__ aux, int3
   if (i < g.N) flag[i] = aux[i] != -2;
 }
 
-// LU with partial pivoting (one CTA), then the explicit inverse, of the leading n x n block
-// (n read on the device) of the stride-ld array Ag; the inverse goes to inv with stride ld.
-// With room for it (smem_elems elements of dynamic shared memory) the matrix, and then also
-// the inverse, are worked on in shared memory (stride n).
+// Panel of one block step: rows k0 .. n - 1 of columns k0 .. k0 + bb - 1, in shared memory column
+// by column; LU with partial pivoting (ties: the lowest row).  Writes the inverse of the pivot
+// block, the row each row of the step comes from and the row order so far.
 template <typename T>
-__global__ void k_coarse_lu(T* __restrict__ Ag, int ld, const int* __restrict__ nu_dev, int aug,
-                            int32_t* __restrict__ piv, T* __restrict__ inv, int* status, size_t smem_elems) {
+__global__ void __launch_bounds__(1024) k_gj_panel(const T* __restrict__ buf, int ld, const int* __restrict__ nu_dev,
+                                                   int aug, int step, int b, int* __restrict__ order,
+                                                   int* __restrict__ from, T* __restrict__ D, int* status) {
   extern __shared__ unsigned char smraw[];
-  __shared__ int s_p;
-  __shared__ T s_best[32];
-  __shared__ int s_bi[32];
-  const int tid = threadIdx.x, nt = blockDim.x;
-  const int nu = *nu_dev + aug;           // the system's dimension (the name of the loops below)
-  if (nu <= 0 || nu > ld) return;         // out of range: reported by k_coarse_assemble
-  const size_t nn = (size_t)nu * nu;
-  const int in_smem = 2 * nn <= smem_elems ? 2 : (nn <= smem_elems ? 1 : 0);
-  const int la = in_smem ? nu : ld;       // stride of the working copy
-  T* A = in_smem ? (T*)smraw : Ag;
-  if (in_smem)
-    for (size_t e = tid; e < nn; e += nt) A[e] = Ag[(e / nu) * ld + e % nu];
+  __shared__ T s_best[2][32];
+  __shared__ int s_row[2][32];
+  const GJView V(nu_dev, aug, ld, b);
+  const int n = V.n, k0 = step * b;
+  if (k0 >= n) return;
+  const int bb = min(b, n - k0), h = n - k0;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  T* P = (T*)smraw;                      // [bb][h]
+  int* rows = (int*)(P + (size_t)bb * h);
+  const T* src = buf + (size_t)V.src(step) * ld * ld;
+  for (int e = tid; e < h * bb; e += 1024) {
+    const int r = e / bb, c = e - r * bb;
+    P[(size_t)c * h + r] = src[(size_t)(k0 + r) * ld + k0 + c];
+  }
+  for (int r = tid; r < h; r += 1024) rows[r] = k0 + r;
   __syncthreads();
-  for (int k = 0; k < nu; ++k) {
-    T best = -1;
-    int bi = k;
-    for (int r = k + tid; r < nu; r += nt) {
-      T v = fabs(A[(size_t)r * la + k]);
-      if (v > best) { best = v; bi = r; }
-    }
+  T best = -1;
+  int row = h;
+  for (int r = tid; r < h; r += 1024) {
+    const T v = fabs(P[r]);
+    if (v > best) { best = v; row = r; }
+  }
+  for (int j = 0; j < bb; ++j) {
     for (int o = 16; o > 0; o >>= 1) {
-      T ob = __shfl_xor_sync(0xffffffffu, best, o);
-      int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-      if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
+      const T ob = __shfl_xor_sync(0xffffffffu, best, o);
+      const int orow = __shfl_xor_sync(0xffffffffu, row, o);
+      if (ob > best || (ob == best && orow < row)) { best = ob; row = orow; }
     }
-    if ((tid & 31) == 0) { s_best[tid >> 5] = best; s_bi[tid >> 5] = bi; }
+    if (lane == 0) { s_best[j & 1][wid] = best; s_row[j & 1][wid] = row; }
     __syncthreads();
-    if (tid < 32) {                     // the warps' candidates, reduced by the first warp
-      T b0 = tid < nt / 32 ? s_best[tid] : (T)-1;
-      int i0 = tid < nt / 32 ? s_bi[tid] : nu;
-      for (int o = 16; o > 0; o >>= 1) {
-        T ob = __shfl_xor_sync(0xffffffffu, b0, o);
-        int oi = __shfl_xor_sync(0xffffffffu, i0, o);
-        if (ob > b0 || (ob == b0 && oi < i0)) { b0 = ob; i0 = oi; }
-      }
-      if (tid == 0) {
-        s_p = i0;
-        piv[k] = i0;
-        if (!(b0 > 0)) set_status(status, IIM_ERR_SINGULAR);
-      }
+    best = s_best[j & 1][lane];          // every warp reduces the warps' candidates
+    row = s_row[j & 1][lane];
+    for (int o = 16; o > 0; o >>= 1) {
+      const T ob = __shfl_xor_sync(0xffffffffu, best, o);
+      const int orow = __shfl_xor_sync(0xffffffffu, row, o);
+      if (ob > best || (ob == best && orow < row)) { best = ob; row = orow; }
     }
-    __syncthreads();
-    const int p = s_p;
-    if (p != k)
-      for (int c = tid; c < nu; c += nt) {
-        T t = A[(size_t)k * la + c];
-        A[(size_t)k * la + c] = A[(size_t)p * la + c];
-        A[(size_t)p * la + c] = t;
+    if (tid == 0 && !(best > 0)) set_status(status, IIM_ERR_SINGULAR);
+    const int p = best >= 0 ? row : j;   // NaN entries only: no candidate
+    if (p != j) {
+      if (tid < bb) {
+        const T t = P[(size_t)tid * h + j];
+        P[(size_t)tid * h + j] = P[(size_t)tid * h + p];
+        P[(size_t)tid * h + p] = t;
+      } else if (tid == 32) {
+        const int t = rows[j];
+        rows[j] = rows[p];
+        rows[p] = t;
       }
-    __syncthreads();
-    const T d = A[(size_t)k * la + k];
-    const int rem = nu - k - 1;
-    for (int r = k + 1 + tid; r < nu; r += nt) A[(size_t)r * la + k] /= d;
-    __syncthreads();
-    for (int e = tid; e < rem * rem; e += nt) {
-      int r = k + 1 + e / rem, c = k + 1 + e % rem;
-      A[(size_t)r * la + c] -= A[(size_t)r * la + k] * A[(size_t)k * la + c];
     }
     __syncthreads();
+    const T d = P[(size_t)j * h + j];
+    best = -1;
+    row = h;
+    for (int r = j + 1 + tid; r < h; r += 1024) {
+      const T l = P[(size_t)j * h + r] / d;
+      P[(size_t)j * h + r] = l;
+      for (int c = j + 1; c < bb; ++c) {
+        const T v = P[(size_t)c * h + r] - l * P[(size_t)c * h + j];
+        P[(size_t)c * h + r] = v;
+        if (c == j + 1 && fabs(v) > best) { best = fabs(v); row = r; }
+      }
+    }
   }
-  if (in_smem)
-    for (size_t e = tid; e < nn; e += nt) Ag[(e / nu) * ld + e % nu] = A[e];
   __syncthreads();
-  if (in_smem == 2) {
-    // inverse in shared memory: X = U^-1 L^-1 P, all columns at once, one row per step.
-    // Column j is handled by G consecutive lanes that split the row's dot product.
-    T* X = A + nn;
-    for (size_t e = tid; e < nn; e += nt) X[e] = 0;
-    __syncthreads();
-    for (int j = tid; j < nu; j += nt) {
-      // P applied to e_j: follow the row swaps in factorisation order
-      int r = j;
-      for (int k = 0; k < nu; ++k) {
-        if (piv[k] == r) r = k;
-        else if (k == r) r = piv[k];
-      }
-      X[(size_t)r * nu + j] = 1;
+  if (wid < bb) {
+    // column wid of (L U)^-1, rows over the lanes
+    T x = lane == wid ? (T)1 : (T)0;
+    for (int i = 0; i < bb; ++i) {
+      const T xi = __shfl_sync(0xffffffffu, x, i);
+      if (lane > i && lane < bb) x -= P[(size_t)i * h + lane] * xi;
     }
-    __syncthreads();
-    int G = 1;
-    while (G < 32 && 2 * G * nu <= nt) G *= 2;
-    const int sub = tid % G, cols = nt / G;
-    for (int r = 1; r < nu; ++r) {                  // forward, unit lower
-      for (int j0 = 0; j0 < nu; j0 += cols) {
-        const int j = j0 + tid / G;
-        T s = 0;
-        if (j < nu)
-          for (int c = sub; c < r; c += G) s += A[(size_t)r * nu + c] * X[(size_t)c * nu + j];
-        for (int o = G / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o, G);
-        if (j < nu && sub == 0) X[(size_t)r * nu + j] -= s;
-      }
-      __syncthreads();
+    for (int i = bb - 1; i >= 0; --i) {
+      const T xi = __shfl_sync(0xffffffffu, x, i) / P[(size_t)i * h + i];
+      if (lane == i) x = xi;
+      else if (lane < i) x -= P[(size_t)i * h + lane] * xi;
     }
-    for (int r = nu - 1; r >= 0; --r) {             // backward
-      for (int j0 = 0; j0 < nu; j0 += cols) {
-        const int j = j0 + tid / G;
-        T s = 0;
-        if (j < nu)
-          for (int c = r + 1 + sub; c < nu; c += G) s += A[(size_t)r * nu + c] * X[(size_t)c * nu + j];
-        for (int o = G / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o, G);
-        if (j < nu && sub == 0) X[(size_t)r * nu + j] = (X[(size_t)r * nu + j] - s) / A[(size_t)r * nu + r];
-      }
-      __syncthreads();
-    }
-    for (size_t e = tid; e < nn; e += nt) inv[(e / nu) * ld + e % nu] = X[e];
-    return;
+    if (lane < bb) D[lane * kGJ + wid] = x;
   }
-  // inverse from the factors in global memory (stride ld): solve L U x = P e_j, one warp per column
-  const int lane = tid & 31, wid = tid >> 5, nw = nt / 32;
-  for (int j = wid; j < nu; j += nw) {
-    T* x = inv + (size_t)j;      // column j of the (row major, stride ld) inverse
-    for (int r = lane; r < nu; r += 32) x[(size_t)r * ld] = (r == j) ? (T)1 : (T)0;
-    __syncwarp();
-    if (lane == 0)
-      for (int k = 0; k < nu; ++k) {
-        int p = piv[k];
-        if (p != k) { T t = x[(size_t)k * ld]; x[(size_t)k * ld] = x[(size_t)p * ld]; x[(size_t)p * ld] = t; }
-      }
-    __syncwarp();
-    for (int r = 0; r < nu; ++r) {                 // forward, unit lower
-      T part = 0;
-      for (int c = lane; c < r; c += 32) part += Ag[(size_t)r * ld + c] * x[(size_t)c * ld];
-      for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-      if (lane == 0) x[(size_t)r * ld] -= part;
-      __syncwarp();
-    }
-    for (int r = nu - 1; r >= 0; --r) {            // backward
-      T part = 0;
-      for (int c = r + 1 + lane; c < nu; c += 32) part += Ag[(size_t)r * ld + c] * x[(size_t)c * ld];
-      for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-      if (lane == 0) x[(size_t)r * ld] = (x[(size_t)r * ld] - part) / Ag[(size_t)r * ld + r];
-      __syncwarp();
-    }
+  for (int r = tid; r < h; r += 1024) from[k0 + r] = rows[r];
+  int old[4];                            // n <= 4096 + 1: at most five rows per thread
+  int last = 0;
+  for (int r = tid, q = 0; r < h; r += 1024, ++q) {
+    const int v = step == 0 ? rows[r] : order[rows[r]];
+    if (q < 4) old[q] = v;
+    else last = v;
   }
+  __syncthreads();
+  for (int r = tid, q = 0; r < h; r += 1024, ++q) order[k0 + r] = q < 4 ? old[q] : last;
+}
+
+// One 32 x 32 tile of a block step.  With A the matrix in the step's row order and K the pivot
+// columns (rows): T = A_KK^-1 A_K: (the inverse itself in the columns K); rows K become T, the
+// others A - A_:K T (minus A_:K T in the columns K).
+template <typename T>
+__global__ void __launch_bounds__(256) k_gj_update(T* __restrict__ buf, int ld, const int* __restrict__ nu_dev, int aug,
+                                                   int step, int b, const int* __restrict__ from,
+                                                   const T* __restrict__ D) {
+  __shared__ T sD[kGJ][kGJ + 1], sK[kGJ][kGJ], sT[kGJ][kGJ], sA[32][kGJ + 1];
+  const GJView V(nu_dev, aug, ld, b);
+  const int n = V.n, k0 = step * b;
+  const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
+  if (k0 >= n || r0 >= n || c0 >= n) return;
+  const int bb = min(b, n - k0);
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const T* src = buf + (size_t)V.src(step) * ld * ld;
+  T* dst = buf + (size_t)(1 - V.src(step)) * ld * ld;
+  const int c = c0 + tx;
+  const bool cK = c >= k0 && c < k0 + bb;
+  T a[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int j = ty + 8 * q, r = r0 + j;
+    const int fr = r < n ? (r < k0 ? r : from[r]) : 0;
+    sD[j][tx] = j < bb && tx < bb ? D[j * kGJ + tx] : (T)0;
+    sK[j][tx] = j < bb && c < n ? src[(size_t)from[k0 + j] * ld + c] : (T)0;
+    sA[j][tx] = r < n && tx < bb ? src[(size_t)fr * ld + k0 + tx] : (T)0;
+    a[q] = r < n && c < n && !cK ? src[(size_t)fr * ld + c] : (T)0;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int j = ty + 8 * q;
+    T s = 0;
+    if (cK) s = sD[j][c - k0];
+    else
+      for (int i = 0; i < bb; ++i) s = fma(sD[j][i], sK[i][tx], s);
+    sT[j][tx] = s;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int j = ty + 8 * q, r = r0 + j;
+    if (r >= n || c >= n) continue;
+    T s = a[q];
+    if (r >= k0 && r < k0 + bb) s = sT[r - k0][tx];
+    else
+      for (int i = 0; i < bb; ++i) s = fma(-sA[j][i], sT[i][tx], s);
+    dst[(size_t)r * ld + c] = s;
+  }
+}
+
+// buffer 0 holds the inverse of the matrix with its rows in the order `order`: its columns go
+// back to the original rows' places
+template <typename T>
+__global__ void __launch_bounds__(256) k_gj_finish(T* __restrict__ buf, int ld, const int* __restrict__ nu_dev, int aug,
+                                                   int b, const int* __restrict__ order) {
+  const GJView V(nu_dev, aug, ld, b);
+  const int c = blockIdx.x * 256 + threadIdx.x;
+  if (c >= V.n) return;
+  const int oc = order[c];
+  for (int r = blockIdx.y; r < V.n; r += gridDim.y) buf[((size_t)ld + r) * ld + oc] = buf[(size_t)r * ld + c];
 }
 
 // ---------------------------------------------------------------------------- host side
@@ -727,7 +768,36 @@ bool mg_one_kernel(Problem& P, int which, const double* v, double* z, cudaStream
   return mg_one_kernel_t<float>(P, which, v, z, s);
 }
 
-// coarse matrix, LU and inverse; coarse_lu{64,32} hold [A (cn*cn) | inverse (cn*cn)], cn the
+// columns per block step: the panel's columns must fit in shared memory
+template <typename T>
+static int gj_block(int cn) {
+  int b = kGJ;
+  while (b > 1 && (sizeof(T) * b + sizeof(int)) * (size_t)cn > 220 * 1024) b /= 2;
+  return b;
+}
+
+// dense matrix and inverse of the coarsest level: buf holds two cn x cn buffers and one pivot block
+template <typename T>
+static void coarse_invert(Problem& P, const LevelView<double>& L, const int* nu, const int32_t* node_row, T* buf,
+                          cudaStream_t s) {
+  const int cn = P.coarse_n, b = gj_block<T>(cn);
+  T* D = buf + 2 * (size_t)cn * cn;
+  int* order = P.coarse_piv;
+  int* from = P.coarse_piv + cn;
+  cudaMemsetAsync(buf, 0, sizeof(T) * 2 * (size_t)cn * cn, s);
+  IIM_LAUNCH(k_coarse_assemble<T>, ceil_div(cn, 64), 64, 0, s, L, P.coarse_map, nu, cn, node_row, buf, P.aug, b,
+             P.d_status);
+  smem_optin((const void*)k_gj_panel<T>);
+  const dim3 tiles(ceil_div(cn, 32), ceil_div(cn, 32));
+  for (int k = 0; k * b < cn; ++k) {
+    const size_t sm = (sizeof(T) * b + sizeof(int)) * (size_t)(cn - k * b);
+    IIM_LAUNCH(k_gj_panel<T>, 1, 1024, sm, s, buf, cn, nu, P.aug, k, b, order, from, D, P.d_status);
+    IIM_LAUNCH(k_gj_update<T>, tiles, 256, 0, s, buf, cn, nu, P.aug, k, b, from, D);
+  }
+  IIM_LAUNCH(k_gj_finish<T>, dim3(ceil_div(cn, 256), std::min(cn, 256)), 256, 0, s, buf, cn, nu, P.aug, b, order);
+}
+
+// coarse matrix and inverse; coarse_lu{64,32} hold [scratch (cn*cn) | inverse (cn*cn) | pivot block], cn the
 // fixed size of the padded system (a re-run set-up with another geometry changes only the
 // device-side unknown count)
 void mg_coarse_factor(Problem& P, cudaStream_t s) {
@@ -742,25 +812,8 @@ void mg_coarse_factor(Problem& P, cudaStream_t s) {
   IIM_LAUNCH(k_coarse_map, ceil_div(C.g.N, Tn), Tn, 0, s, C.g, C.aux, C.idx, P.coarse_map, inv);
   LevelView<double> V = view<double>(C);
   const int* nu = P.d_counts + kCountCoarse;
-  // dynamic shared memory of the factorisation: room for the matrix and its inverse at the
-  // unknown count of the creation's geometry with a quarter more (a later set-up with more
-  // unknowns than that works on them in global memory instead); never more than the padded
-  // system or 200 KB, so that small factorisations leave the SM to other kernels
-  auto factor = [&](auto* A, auto* kernel, size_t esz) {
-    const size_t nb = std::min((size_t)cn, (size_t)P.coarse_nu + P.coarse_nu / 4 + 8 + P.aug);
-    size_t sm = std::min((size_t)2 * nb * nb * esz, (size_t)200 * 1024);
-    smem_optin((const void*)kernel);
-    IIM_LAUNCH(kernel, 1, 1024, sm, s, A, cn, nu, P.aug, P.coarse_piv, A + (size_t)cn * cn, P.d_status, sm / esz);
-  };
-  if (P.opt.mg_precision == IIM_MG_FP64) {
-    IIM_LAUNCH(k_coarse_assemble<double>, ceil_div(cn, 128), 128, 0, s, V, P.coarse_map, nu, cn, inv, P.coarse_lu64,
-               P.aug, P.d_status);
-    factor(P.coarse_lu64, k_coarse_lu<double>, sizeof(double));
-  } else {
-    IIM_LAUNCH(k_coarse_assemble<float>, ceil_div(cn, 128), 128, 0, s, V, P.coarse_map, nu, cn, inv, P.coarse_lu32,
-               P.aug, P.d_status);
-    factor(P.coarse_lu32, k_coarse_lu<float>, sizeof(float));
-  }
+  if (P.opt.mg_precision == IIM_MG_FP64) coarse_invert(P, V, nu, inv, P.coarse_lu64, s);
+  else coarse_invert(P, V, nu, inv, P.coarse_lu32, s);
 }
 
 
