@@ -434,7 +434,7 @@ iim_status iim_problem_create(const iim_problem_desc* desc, const iim_options* o
     Level& L = P.lv[l];
     L.n_irr = read_count(P, 2 + (int)l);
     L.irr_cap = L.n_irr + L.n_irr / 4 + 64;
-    const int D = 2 * d + 1;
+    const int D = sw_row(d);
     IIM_ALLOC(L.irr_node, int32_t, L.irr_cap);
     IIM_ALLOC(L.tab64, double, (size_t)L.irr_cap * D);
     IIM_ALLOC(L.tab32, float, (size_t)L.irr_cap * D);

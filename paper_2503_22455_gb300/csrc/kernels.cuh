@@ -17,12 +17,14 @@ struct GridView {
 // One Shortley-Weller level (Sec. 3.1): aux[i] = -2 (not an unknown), -1 (regular
 // unknown: standard 2d+1 point stencil), k >= 0 (irregular unknown, row k of the table).
 // Table rows hold (diag, c[-x0], c[+x0], c[-x1], c[+x1], [c[-x2], c[+x2]]) of the
-// homogeneous SW operator scaled by 1/h^2.
+// homogeneous SW operator scaled by 1/h^2.  Rows are 5 (2D) or 8 (3D, the last entry 1 / diag; a
+// row is one aligned 32-byte piece in FP32) entries apart.
+__host__ __device__ constexpr int sw_row(int dim) { return dim == 2 ? 5 : 8; }
 struct Level {
   GridView g;
   uint8_t* phase = nullptr;
   int32_t* aux = nullptr;
-  uint8_t* cls = nullptr;         // per node: 1 unknown, 2 irregular row, 4 phase + (red-black tile kernels)
+  uint8_t* cls = nullptr;         // per node: 1 unknown, 2 irregular row, 4 phase +, 8 irregular for the box alone (red-black kernels)
   int32_t* flag = nullptr;        // scratch for the irregular-node scan
   int32_t* idx = nullptr;
   int n_irr = 0, irr_cap = 0;

@@ -66,6 +66,12 @@ template <typename T>
 __device__ __forceinline__ T irr_offdiag(T c1, T c2, T c3, T c4, T l, T r, T d, T u) {
   return fma(c4, u, fma(c3, d, fma(c2, r, mul_rn(c1, l))));
 }
+// 3D: f minus the off-diagonal part of a row (weights and values in the order -x, +x, -y, +y, -z, +z);
+// times the reciprocal diagonal it is the Gauss-Seidel value, minus diag u the residual
+template <typename T>
+__device__ __forceinline__ T off_residual3(T f, T c1, T c2, T c3, T c4, T c5, T c6, T l, T r, T d, T u, T b, T t) {
+  return fma(-c6, t, fma(-c5, b, fma(-c4, u, fma(-c3, d, fma(-c2, r, fma(-c1, l, f))))));
+}
 // residual of a regular cell, f - (dreg u + ih2 s)
 template <typename T>
 __device__ __forceinline__ T res_regular(T f, T u, T s, T dreg, T ih2) { return f - fma(dreg, u, mul_rn(ih2, s)); }
@@ -73,6 +79,25 @@ __device__ __forceinline__ T res_regular(T f, T u, T s, T dreg, T ih2) { return 
 template <typename T>
 __device__ __forceinline__ T prolong_bilinear(T e0, T e1, T e2, T e3) {
   return fma((T)0.0625, e3, fma((T)0.1875, e2, fma((T)0.1875, e1, mul_rn((T)0.5625, e0))));
+}
+
+// trilinear weights; e[k]: k bit 0 the x neighbour's, bit 1 the y neighbour's, bit 2 the z neighbour's side
+template <typename T>
+__device__ __forceinline__ T prolong_trilinear(const T (&e)[8]) {
+  const T w[4] = {(T)0.421875, (T)0.140625, (T)0.046875, (T)0.015625};
+  T a = mul_rn(w[0], e[0]);
+#pragma unroll
+  for (int k = 1; k < 8; ++k) a = fma(w[(k & 1) + ((k >> 1) & 1) + (k >> 2)], e[k], a);
+  return a;
+}
+// Neumann: the mean of the in-domain coarse neighbours (bits of ok)
+template <typename T>
+__device__ __forceinline__ T prolong_mean8(const T (&e)[8], unsigned ok) {
+  T a = 0;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) a += (ok >> k) & 1u ? e[k] : (T)0;
+  const int cnt = __popc(ok & 255u);
+  return cnt > 0 ? a / (T)cnt : (T)0;
 }
 
 template <typename T>
@@ -332,7 +357,7 @@ struct TailParams {
 };
 
 template <typename T>
-__device__ inline T tabd(const T* tb, int dim, int r, int k) { return tb[r * (2 * dim + 1) + k]; }
+__device__ inline T tabd(const T* tb, int dim, int r, int k) { return tb[r * sw_row(dim) + k]; }
 
 // offdiagonal part of (L u)_i from shared-memory u; m = (i0, i1, i2)
 template <typename T, int DIM>
@@ -399,7 +424,7 @@ __device__ __forceinline__ void vcycle_tail_body(const TailParams<T>& P, const d
   if (P.stage_tables) {
     for (int k = 0; k < P.nlev; ++k) {
       const int rows = min(*P.tcount[k], P.tcap[k]);
-      const int len = rows * (2 * DIM + 1);
+      const int len = rows * sw_row(DIM);
       for (int e = tid; e < len; e += nt) st[P.toff[k] + e] = P.L[k].tab[e];
     }
   }

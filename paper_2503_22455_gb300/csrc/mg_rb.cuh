@@ -43,6 +43,7 @@ constexpr int kRbIrrCap = 320;            // staged irregular rows per tile
 
 // cell classes (one byte per node and level)
 constexpr uint8_t kClsUnknown = 1, kClsIrregular = 2, kClsPlus = 4;
+constexpr uint8_t kClsBox = 8;            // irregular for a box face alone: every neighbour on the grid is in phase
 
 template <typename T>
 struct Rb2DParams {

@@ -8,10 +8,12 @@
 // problems run on lap(u) = f/beta per phase (Sec. 3.3): the FP64 Krylov vector
 // is divided by beta_sigma when it enters the FP32 hierarchy.
 #include <algorithm>
+#include <type_traits>
 #include <utility>
 
 #include "engine.cuh"
 #include "mg_rb.cuh"
+#include "mg_3d.cuh"
 
 namespace iim {
 
@@ -24,7 +26,7 @@ struct LevelView {
 
 template <typename T>
 __device__ inline T tabv(const LevelView<T>& L, int r, int k) {
-  return L.tab[(size_t)r * (2 * L.g.dim + 1) + k];
+  return L.tab[(size_t)r * sw_row(L.g.dim) + k];
 }
 
 __device__ inline void idx3(const GridView& g, int64_t i, int* m) {
@@ -34,25 +36,41 @@ __device__ inline void idx3(const GridView& g, int64_t i, int* m) {
   m[2] = g.dim > 2 ? (int)(r / g.n) : 0;
 }
 
-// (L u)_i without the diagonal term: sum of off-diagonal coefficients times neighbours
+// the neighbours' values (-x, +x, -y, +y, -z, +z), zero beyond the grid
 template <typename T>
-__device__ inline T offdiag_sum(const LevelView<T>& L, T ih2, int64_t i, const int* m, int a, const T* __restrict__ u) {
-  const GridView& g = L.g;
-  T s = 0;
-  if (a == -1) {
-    for (int ax = 0; ax < g.dim; ++ax) {
-      int64_t st = ax == 0 ? 1 : (ax == 1 ? (int64_t)g.n : (int64_t)g.n * g.n);
-      s += u[i - st] + u[i + st];
-    }
-    return s * ih2;
+__device__ inline void neighbours(const GridView& g, int64_t i, const int* m, const T* __restrict__ u, T (&v)[6]) {
+#pragma unroll
+  for (int ax = 0; ax < 3; ++ax) {
+    const int64_t st = ax == 0 ? 1 : (ax == 1 ? (int64_t)g.n : (int64_t)g.n * g.n);
+    v[2 * ax] = ax < g.dim && m[ax] > 0 ? u[i - st] : (T)0;
+    v[2 * ax + 1] = ax < g.dim && m[ax] < g.n - 1 ? u[i + st] : (T)0;
   }
-  for (int ax = 0; ax < g.dim; ++ax) {
-    int64_t st = ax == 0 ? 1 : (ax == 1 ? (int64_t)g.n : (int64_t)g.n * g.n);
-    T cl = tabv(L, a, 1 + 2 * ax), cr = tabv(L, a, 2 + 2 * ax);
-    if (cl != (T)0 && m[ax] > 0) s += cl * u[i - st];
-    if (cr != (T)0 && m[ax] < g.n - 1) s += cr * u[i + st];
-  }
-  return s;
+}
+
+// Gauss-Seidel value and residual of a node (aux code a) in the arithmetic of the fused kernels.  3D:
+// every node is a row of weights (ih2 in a regular one) with the diagonal's reciprocal.
+template <typename T>
+__device__ inline T off_residual_node(const LevelView<T>& L, T ih2, int a, T f, const T (&v)[6]) {
+  if (a == -1) return off_residual3(f, ih2, ih2, ih2, ih2, ih2, ih2, v[0], v[1], v[2], v[3], v[4], v[5]);
+  return off_residual3(f, tabv(L, a, 1), tabv(L, a, 2), tabv(L, a, 3), tabv(L, a, 4), tabv(L, a, 5), tabv(L, a, 6), v[0],
+                       v[1], v[2], v[3], v[4], v[5]);
+}
+template <typename T>
+__device__ inline T irregular_sum2(const LevelView<T>& L, int a, const T (&v)[6]) {
+  return irr_offdiag(tabv(L, a, 1), tabv(L, a, 2), tabv(L, a, 3), tabv(L, a, 4), v[0], v[1], v[2], v[3]);
+}
+template <typename T>
+__device__ inline T gs_node(const LevelView<T>& L, T ih2, T inv_dreg, int a, T f, const T (&v)[6]) {
+  if (L.g.dim > 2) return mul_rn(off_residual_node(L, ih2, a, f, v), a == -1 ? inv_dreg : tabv(L, a, 7));
+  if (a == -1) return gs_regular(f, (v[0] + v[1]) + (v[2] + v[3]), ih2, inv_dreg);
+  const T dg = tabv(L, a, 0);
+  return dg != (T)0 ? (f - irregular_sum2(L, a, v)) / dg : (T)0;
+}
+template <typename T>
+__device__ inline T residual_node(const LevelView<T>& L, T ih2, T dreg, int a, T f, T u, const T (&v)[6]) {
+  if (L.g.dim > 2) return fma(-(a == -1 ? dreg : tabv(L, a, 0)), u, off_residual_node(L, ih2, a, f, v));
+  if (a != -1) return f - fma(tabv(L, a, 0), u, irregular_sum2(L, a, v));
+  return res_regular(f, u, (v[0] + v[1]) + (v[2] + v[3]), dreg, ih2);
 }
 
 template <typename T>
@@ -62,7 +80,7 @@ __device__ inline T diag_of(const LevelView<T>& L, T dreg, int a) {
 }
 
 template <typename T>
-__device__ __forceinline__ void smooth_body(const LevelView<T>& L, T ih2, T dreg, T* __restrict__ u,
+__device__ __forceinline__ void smooth_body(const LevelView<T>& L, T ih2, T inv_dreg, T* __restrict__ u,
                                             const T* __restrict__ f, int f_bf16, int colour, int64_t t) {
   // one thread per node of the colour: node = 2 * t + parity fix-up along x
   const GridView& g = L.g;
@@ -78,15 +96,15 @@ __device__ __forceinline__ void smooth_body(const LevelView<T>& L, T ih2, T dreg
   int a = L.aux[i];
   if (a == -2) return;
   int m[3] = {xi, ry, rz};
-  T dg = diag_of(L, dreg, a);
-  T s = offdiag_sum(L, ih2, i, m, a, u);
-  u[i] = dg != (T)0 ? (load_f(f, i, f_bf16) - s) / dg : (T)0;
+  T v[6];
+  neighbours(g, i, m, u, v);
+  u[i] = gs_node(L, ih2, inv_dreg, a, load_f(f, i, f_bf16), v);
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) k_smooth(LevelView<T> L, T ih2, T dreg, T* __restrict__ u,
+__global__ void __launch_bounds__(256) k_smooth(LevelView<T> L, T ih2, T inv_dreg, T* __restrict__ u,
                                                 const T* __restrict__ f, int f_bf16, int colour) {
-  smooth_body<T>(L, ih2, dreg, u, f, f_bf16, colour, (int64_t)blockIdx.x * blockDim.x + threadIdx.x);
+  smooth_body<T>(L, ih2, inv_dreg, u, f, f_bf16, colour, (int64_t)blockIdx.x * blockDim.x + threadIdx.x);
 }
 
 // coarse f = mean over the 2^d children of r = f - L u (zero at non-unknowns)
@@ -100,17 +118,22 @@ __device__ __forceinline__ void resid_restrict_body(const LevelView<T>& F, T ih2
   int mc[3];
   idx3(gc, I, mc);
   const GridView& g = F.g;
-  T acc = 0;
-  const int nch = 1 << g.dim;
-  for (int c = 0; c < nch; ++c) {
+  // rows first, then the two rows of a plane, then the planes
+  T r[8];
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    r[c] = (T)0;
+    if (c >= (1 << g.dim)) continue;
     int m[3] = {2 * mc[0] + (c & 1), 2 * mc[1] + ((c >> 1) & 1), g.dim > 2 ? 2 * mc[2] + ((c >> 2) & 1) : 0};
     int64_t i = m[0] + (int64_t)g.n * m[1] + (int64_t)g.n * g.n * m[2];
     int a = F.aux[i];
     if (a == -2) continue;
-    T r = load_f(f, i, f_in_bf16) - (diag_of(F, dreg, a) * u[i] + offdiag_sum(F, ih2, i, m, a, u));
-    acc += r;
+    T v[6];
+    neighbours(g, i, m, u, v);
+    r[c] = residual_node(F, ih2, dreg, a, load_f(f, i, f_in_bf16), u[i], v);
   }
-  store_f(fc, I, acc / (T)nch, f_bf16);
+  const T lo = (r[0] + r[1]) + (r[2] + r[3]);
+  store_f(fc, I, g.dim > 2 ? (lo + ((r[4] + r[5]) + (r[6] + r[7]))) * (T)0.125 : lo * (T)0.25, f_bf16);
 }
 
 template <typename T>
@@ -133,29 +156,26 @@ __device__ __forceinline__ void prolong_body(const GridView& gf, const int32_t* 
   idx3(gf, i, m);
   int I[3] = {m[0] >> 1, m[1] >> 1, m[2] >> 1};
   int sg[3] = {(m[0] & 1) ? 1 : -1, (m[1] & 1) ? 1 : -1, (m[2] & 1) ? 1 : -1};
-  T acc = 0;
-  int cnt = 0;
-  const int nsel = 1 << gf.dim;
-  for (int sel = 0; sel < nsel; ++sel) {
+  T ev[8];
+  unsigned ok = 0;
+#pragma unroll
+  for (int sel = 0; sel < 8; ++sel) {
+    ev[sel] = (T)0;
+    if (sel >= (1 << gf.dim)) continue;
     int c[3];
-    T wgt = 1;
     bool inb = true;
     for (int k = 0; k < 3; ++k) {
-      int b = (sel >> k) & 1;
-      c[k] = k < gf.dim ? I[k] + b * sg[k] : 0;
-      if (k < gf.dim) {
-        if (c[k] < 0 || c[k] >= gc.n) inb = false;
-        wgt *= b ? (T)0.25 : (T)0.75;
-      }
+      c[k] = k < gf.dim ? I[k] + ((sel >> k) & 1) * sg[k] : 0;
+      if (k < gf.dim && (c[k] < 0 || c[k] >= gc.n)) inb = false;
     }
     if (!inb) continue;
     int64_t ci = c[0] + (int64_t)gc.n * c[1] + (int64_t)gc.n * gc.n * c[2];
     if (aux_c[ci] == -2) continue;
-    if (neumann) { acc += ec[ci]; ++cnt; }
-    else acc += wgt * ec[ci];
+    ev[sel] = ec[ci];
+    ok |= 1u << sel;
   }
-  if (neumann) acc = cnt > 0 ? acc / (T)cnt : (T)0;
-  uf[i] += acc;
+  uf[i] += neumann ? prolong_mean8(ev, ok)
+                   : (gf.dim > 2 ? prolong_trilinear(ev) : prolong_bilinear(ev[0], ev[1], ev[2], ev[3]));
 }
 
 template <typename T>
@@ -173,8 +193,7 @@ __device__ __forceinline__ void bridge_in_body(const GridView& g, const double* 
                                                T* __restrict__ f, int64_t i) {
   if (i >= g.N) return;
   if (aux[i] == -2) { f[i] = (T)0; return; }
-  const T sc = (T)((scale ? *scale : 1.0) * (phase[i] ? inv_bp : inv_bm));
-  f[i] = (T)v[i] * sc;
+  f[i] = mul_rn((T)v[i], mul_rn((T)(scale ? *scale : 1.0), (T)(phase[i] ? inv_bp : inv_bm)));
 }
 
 template <typename T>
@@ -477,7 +496,7 @@ TailParams<T> make_tail_params(Problem& P, size_t l0, T* u_out, size_t smem_limi
     tp.toff[k] = toff;
     tp.tcount[k] = P.d_counts + 2 + (int)(l0 + k);
     tp.tcap[k] = L.irr_cap;
-    toff += L.irr_cap * (2 * L.g.dim + 1);
+    toff += L.irr_cap * sw_row(L.g.dim);
   }
   tp.toff[tp.nlev] = toff;
   const size_t base = (sizeof(T) * 2 + 2 * sizeof(int)) * (size_t)off;   // u, f, aux, node coordinates
@@ -670,7 +689,91 @@ static T* vcycle2d(Problem& P, size_t l, size_t lt, const double* v, const doubl
   return B;
 }
 
-// generic path (3D fine levels): one kernel per half sweep, transfers separate; u is
+template <typename T>
+static Grid3D<T> grid3d(const Level& L) {
+  const LevelK<T> K = levk<T>(L);
+  Grid3D<T> G;
+  G.n = L.g.n;
+  G.ih2 = K.ih2;
+  G.inv_dreg = K.inv_dreg;
+  G.dreg = K.dreg;
+  // rows of nodes at box faces, as k_sw_fill computes them (a face half a cell away: psi = 1/2)
+  const double h2 = L.g.h * L.g.h;
+  G.wall = (T)(2.0 / (1.0 * (0.5 + 1.0)) / h2);
+  for (int k = 0; k < 4; ++k) {
+    double d = 0;
+    for (int ax = 0; ax < 3; ++ax) d += ax < k ? -2.0 / (0.5 * 1.0) / h2 : -2.0 / (1.0 * 1.0) / h2;
+    G.wdiag[k] = (T)d;
+    G.winv[k] = (T)(1.0 / d);
+  }
+  G.cls = L.cls;
+  G.aux = L.aux;
+  G.tab = K.tab;
+  return G;
+}
+
+// Planes per thread of a half sweep: 16 on the levels whose u and f take more than half of L2
+// (256^3: 51 -> 41 us per half sweep); one below, where the loop only adds latency (128^3: 9.6 us
+// against 10.7 with runs of 4).
+static int smooth3d_run(int n) { return (int64_t)n * n * n * 8 > (64 << 20) ? 16 : 1; }
+
+// 3D: u of every level is updated in place (stored by colour above the tail) and starts from zero unless this is a later visit of a
+// W-cycle.  The level's right-hand side is v scale / beta on the finest level (v set), else L.f; the
+// finest level's result leaves through z.
+template <typename T>
+static void vcycle3d(Problem& P, size_t l, size_t lt, const double* v, const double* vscale, double* z, cudaStream_t s,
+                     bool from_zero = true) {
+  Level& L = P.lv[l];
+  T* u = (T*)L.u;
+  T* f = (T*)L.f;
+  if (l == lt) {
+    launch_tail<T>(P, l, nullptr, nullptr, nullptr, s);
+    return;
+  }
+  const int Tn = 256, n = L.g.n;
+  const Grid3D<T> G = grid3d<T>(L);
+  const dim3 grid(ceil_div(n * (n / 2), Tn), n);
+  const int run = smooth3d_run(n);
+  const dim3 grid_s(grid.x, ceil_div(n, run));
+  auto sweep = [&](int colour, bool out) {
+    if (out) IIM_LAUNCH_PDL((k_smooth3d<T, true>), grid_s, Tn, 0, s, G, u, (const T*)f, L.f_bf16, colour, run, z);
+    else IIM_LAUNCH_PDL((k_smooth3d<T, false>), grid_s, Tn, 0, s, G, u, (const T*)f, L.f_bf16, colour, run, (double*)nullptr);
+  };
+  if (from_zero)
+    IIM_LAUNCH_PDL(k_first3d<T>, grid, Tn, 0, s, G, v, vscale, (T)(1.0 / P.desc.beta_plus), (T)(1.0 / P.desc.beta_minus),
+                   f, L.f_bf16, u);
+  for (int it = 0; it < P.opt.nu1; ++it)
+    for (int c = 0; c < 2; ++c)
+      if (!(from_zero && it == 0 && c == 0)) sweep(c, false);
+  Level& C = P.lv[l + 1];
+  const int nc = C.g.n;
+  const bool split = l + 1 < lt;         // the tail's levels keep the natural order
+  auto transfers = [&](auto split_, auto rows_, bool down) {
+    constexpr int SPLIT = decltype(split_)::value, ROWS = decltype(rows_)::value;
+    const dim3 grid_c(ceil_div(4 / ROWS * nc * nc, Tn), nc);
+    if (down)
+      IIM_LAUNCH_PDL((k_restrict3d<T, SPLIT, ROWS>), grid_c, Tn, 0, s, G, (const T*)u, (const T*)f, L.f_bf16, nc,
+                     (const uint8_t*)C.cls, (T*)C.f, C.f_bf16);
+    else
+      IIM_LAUNCH_PDL((k_prolong3d<T, SPLIT, ROWS>), grid_c, Tn, 0, s, n, (const uint8_t*)L.cls, u, nc, (const uint8_t*)C.cls,
+                     (const T*)C.u, (int)(P.desc.bc == IIM_BC_NEUMANN));
+  };
+  auto transfer = [&](bool down) {
+    using std::integral_constant;
+    if (!split) transfers(integral_constant<int, 0>(), integral_constant<int, 1>(), down);
+    else if (n < 128) transfers(integral_constant<int, 1>(), integral_constant<int, 1>(), down);
+    else transfers(integral_constant<int, 1>(), integral_constant<int, 4>(), down);
+  };
+  transfer(true);
+  if (l + 1 == lt) vcycle3d<T>(P, l + 1, lt, nullptr, nullptr, nullptr, s);
+  else
+    for (int g = 0; g < P.opt.cycle; ++g) vcycle3d<T>(P, l + 1, lt, nullptr, nullptr, nullptr, s, g == 0);
+  transfer(false);
+  for (int it = 0; it < P.opt.nu2; ++it)
+    for (int c = 0; c < 2; ++c) sweep(c, z != nullptr && it == P.opt.nu2 - 1 && c == 1);
+}
+
+// generic path (2D with fewer than two sweeps): one kernel per half sweep, transfers separate; u is
 // updated in place and starts from zero unless this is a later visit of a W-cycle
 template <typename T>
 static void vcycle(Problem& P, size_t l, size_t lt, cudaStream_t s, bool from_zero = true) {
@@ -688,7 +791,7 @@ static void vcycle(Problem& P, size_t l, size_t lt, cudaStream_t s, bool from_ze
   if (from_zero) IIM_LAUNCH(k_zero<T>, ceil_div(L.g.N, Tn), Tn, 0, s, u, L.g.N);
   for (int it = 0; it < P.opt.nu1; ++it)
     for (int c = 0; c < 2; ++c)
-      IIM_LAUNCH(k_smooth<T>, ceil_div(ncol, Tn), Tn, 0, s, V, K.ih2, K.dreg, u, f, L.f_bf16, c);
+      IIM_LAUNCH(k_smooth<T>, ceil_div(ncol, Tn), Tn, 0, s, V, K.ih2, K.inv_dreg, u, f, L.f_bf16, c);
   Level& C = P.lv[l + 1];
   IIM_LAUNCH(k_resid_restrict<T>, ceil_div(C.g.N, Tn), Tn, 0, s, V, K.ih2, K.dreg, u, f, L.f_bf16, C.g, C.aux,
              (T*)C.f, C.f_bf16);
@@ -699,7 +802,7 @@ static void vcycle(Problem& P, size_t l, size_t lt, cudaStream_t s, bool from_ze
              P.desc.bc == IIM_BC_NEUMANN);
   for (int it = 0; it < P.opt.nu2; ++it)
     for (int c = 0; c < 2; ++c)
-      IIM_LAUNCH(k_smooth<T>, ceil_div(ncol, Tn), Tn, 0, s, V, K.ih2, K.dreg, u, f, L.f_bf16, c);
+      IIM_LAUNCH(k_smooth<T>, ceil_div(ncol, Tn), Tn, 0, s, V, K.ih2, K.inv_dreg, u, f, L.f_bf16, c);
 }
 
 template <typename T>
@@ -715,6 +818,10 @@ static void precondition_t(Problem& P, const double* v, const double* vscale, do
     vcycle2d<T>(P, 0, lt, v, vscale, z, s);
     return;
   }
+  if (P.g.dim == 3 && P.opt.nu1 >= 1 && P.opt.nu2 >= 1) {
+    vcycle3d<T>(P, 0, lt, v, vscale, z, s);
+    return;
+  }
   IIM_LAUNCH(k_bridge_in<T>, ceil_div(L.g.N, Tn), Tn, 0, s, L.g, v, vscale, P.phase, L.aux,
              1.0 / P.desc.beta_plus, 1.0 / P.desc.beta_minus, (T*)L.f);
   vcycle<T>(P, 0, lt, s);
@@ -724,10 +831,17 @@ static void precondition_t(Problem& P, const double* v, const double* vscale, do
 template <typename T>
 static void smooth_fine_t(Problem& P, int colour, cudaStream_t s) {
   Level& L = P.lv[0];
+  if (P.g.dim == 3 && tail_start(P) > 0) {
+    const int n = L.g.n;
+    const int run = smooth3d_run(n);
+    IIM_LAUNCH_PDL((k_smooth3d<T, false>), dim3(ceil_div(n * (n / 2), 256), ceil_div(n, run)), 256, 0, s, grid3d<T>(L),
+                   (T*)L.u, (const T*)L.f, L.f_bf16, colour, run, (double*)nullptr);
+    return;
+  }
   LevelView<T> V = view<T>(L);
   LevelK<T> K = levk<T>(L);
   const int64_t ncol = (L.g.N / L.g.n) * ((L.g.n + 1) / 2);
-  IIM_LAUNCH(k_smooth<T>, ceil_div(ncol, 256), 256, 0, s, V, K.ih2, K.dreg, (T*)L.u, (const T*)L.f, L.f_bf16, colour);
+  IIM_LAUNCH(k_smooth<T>, ceil_div(ncol, 256), 256, 0, s, V, K.ih2, K.inv_dreg, (T*)L.u, (const T*)L.f, L.f_bf16, colour);
 }
 
 // one red or black half sweep on the finest level (kernel timing)
@@ -893,7 +1007,7 @@ __global__ void __launch_bounds__(256) k_eng_mg3d(EngArgs A, int list, int d, in
     } else if (KIND == 1) {
       if (i < K.N) K.u[i] = 0.f;
     } else if (KIND == 2) {
-      smooth_body<float>(V, K.ih2, K.dreg, K.u, K.f, K.f_bf16, colour, i);
+      smooth_body<float>(V, K.ih2, K.inv_dreg, K.u, K.f, K.f_bf16, colour, i);
     } else if (KIND == 3) {
       const LevelView<float> C = eng_view(s, d + 1);
       resid_restrict_body<float>(V, K.ih2, K.dreg, K.u, K.f, K.f_bf16, C.g, C.aux, s.lev[d + 1].f, i,

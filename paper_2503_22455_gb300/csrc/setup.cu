@@ -532,13 +532,17 @@ __global__ void k_sw_classify(SWParams P, const uint8_t* __restrict__ phase, int
   } else {
     int m[3];
     node_index(g, i, m);
+    int cut = 0;                       // a neighbour on the grid is out of phase
     for (int ax = 0; ax < g.dim; ++ax)
       for (int s = -1; s <= 1; s += 2) {
         int pos = m[ax] + s;
-        if (pos < 0 || pos >= g.n || phase[i + s * stride_of(g, ax)] != phase[i]) f = 1;
+        if (pos < 0 || pos >= g.n) f = 1;
+        else if (phase[i + s * stride_of(g, ax)] != phase[i]) cut = 1;
       }
+    // unknown, and irregular (its row is filled by k_sw_fill), for the box alone or not
+    c |= cut ? 3 : (f ? 11 : 1);
+    f |= cut;
     aux[i] = -1;
-    c |= f ? 3 : 1;                    // unknown, and irregular: its row is filled by k_sw_fill
   }
   cls[i] = c;
   flag[i] = f;
@@ -554,7 +558,7 @@ __global__ void k_sw_fill(SWParams P, const uint8_t* __restrict__ phase, const i
   const int64_t i = list[r];
   int m[3];
   node_index(g, i, m);
-  const int D = 2 * g.dim + 1;
+  const int D = sw_row(g.dim);
   const double h2 = g.h * g.h;
   // interface wall weights (homogeneous Eq. 21, psi = 1/2): uw = lam_m u(minus node) + lam_p u(plus node)
   const double am = 0.5 / P.beta_m, ap = 0.5 / P.beta_p;
@@ -594,6 +598,11 @@ __global__ void k_sw_fill(SWParams P, const uint8_t* __restrict__ phase, const i
   for (int k = 0; k < 2 * g.dim; ++k) {
     tab64[(size_t)r * D + 1 + k] = off[k];
     tab32[(size_t)r * D + 1 + k] = (float)off[k];
+  }
+  if (g.dim > 2) {                       // 3D rows carry the reciprocal diagonal in their last entry
+    const double inv = diag != 0.0 ? 1.0 / diag : 0.0;
+    tab64[(size_t)r * D + 7] = inv;
+    tab32[(size_t)r * D + 7] = (float)inv;
   }
   aux[i] = r;
 }
