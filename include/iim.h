@@ -440,7 +440,7 @@ iim_status iim_gradient(iim_problem* p, const double* u_dev, double* grad_dev);
 /* Profiling: average device time (microseconds) of one launch of an internal
  * kernel, timed with CUDA events on the problem's stream over ``reps`` back to
  * back launches on the problem's own vectors (after 3 untimed launches).
- * which: 0 high-order stencil, 1 ghost values, 2 corrections (Eq. 12 operator
+ * which: 0 plain nodes, 1 ghost values, 2 affected nodes (Eq. 12 operator
  * kernels); 3 one red half sweep on the finest level; 4 FGMRES multi-dot and
  * 5 update over restart/2 + 1 vectors; 6 a whole V-cycle; 7 the whole operator;
  * 8 the least-squares fits of the set-up (Sec. 2.1-2.2); 9 / 10 the first level's fused

@@ -340,6 +340,9 @@ iim_status iim_problem_create(const iim_problem_desc* desc, const iim_options* o
   IIM_ALLOC(P.edge_flag, int32_t, N * d);
   IIM_ALLOC(P.edge_id, int32_t, N * d);
   IIM_ALLOC(P.aff_flag, int32_t, N);
+  // the edge flags are done with when the nodes are classed: their memory (4 d N bytes) holds the classes
+  P.kind = (uint8_t*)P.edge_flag;
+  P.tile_kind = P.kind + N;                // less than N of them
   IIM_ALLOC(P.aff_idx, int32_t, N);
   P.scan_scratch_len = scan_scratch_ints(N * d) + 64;
   IIM_ALLOC(P.scan_scratch, int, P.scan_scratch_len);
@@ -908,9 +911,9 @@ iim_status iim_kernel_time_flushed(iim_problem* H, int which, int reps, void* fl
   const int j = P.opt.restart / 2;
   auto launch = [&]() {
     switch (which) {
-      case 0: ho_stencil(P, P.x, P.tmp, s); break;
-      case 1: ho_ghost(P, P.x, false, s); break;
-      case 2: ho_correct(P, P.x, P.tmp, false, s); break;
+      case 0: ho_nodes(P, P.x, P.tmp, false, P.G, 1, s); break;
+      case 1: ho_ghost(P, P.x, false, P.G, s); break;
+      case 2: ho_nodes(P, P.x, P.tmp, false, P.G, 2, s); break;
       case 3: mg_smooth_fine(P, 0, s); break;
       case 4: krylov_orth_pass(P, j, 0, s); break;
       case 5: krylov_orth_pass(P, j, 1, s); break;

@@ -108,6 +108,8 @@ static void fill_slot(Engine& E, int si, Problem& P) {
   sd.neumann = P.desc.bc == IIM_BC_NEUMANN;
   sd.g = P.g;
   sd.phase = P.phase;
+  sd.kind = P.kind;
+  sd.tile_kind = P.tile_kind;
   sd.status = P.d_status + 1;           // the per-solve word (set-up failures stay in word 0)
   eng_operator_params(P, &sd.C, &sd.GP, &sd.CP);
   sd.sc = P.sc;
@@ -144,7 +146,9 @@ static void build_lists(Engine& E) {
     L[kListAll].push_back({si, 1});
     L[kListXup].push_back({si, sd.xup_blocks});
     L[kListRed].push_back({si, sd.red_blocks});
-    L[kListStencil + (P.g.dim - 2) * 2 + (P.w - 2)].push_back({si, cdiv(P.g.N, 4 * kEngThreads)});
+    const int tiles = op_tile_count(P);
+    if (tiles > 0) L[kListTile].push_back({si, tiles});
+    else L[kListStencil + (P.g.dim - 2) * 2 + (P.w - 2)].push_back({si, cdiv(P.g.N, 4 * kEngThreads)});
     if (P.K_cap > 0) L[kListGhost + (P.w - 2)].push_back({si, cdiv((int64_t)P.K_cap * 8, 64)});
     if (P.aff_cap > 0) L[kListCorrect].push_back({si, cdiv(P.aff_cap, 64)});
     L[kListTail].push_back({si, 1});

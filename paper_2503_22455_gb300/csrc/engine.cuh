@@ -36,7 +36,8 @@ enum EngList {
   kListXup,                                    // x += Z y
   kListRed,                                    // reductions: red_blocks items
   kListStencil,                                // + (dim - 2) * 2 + (w - 2): four lists
-  kListGhost = kListStencil + 4,               // + (w - 2): two lists
+  kListTile = kListStencil + 4,                // problems with fixed-point tiles (3D, order 4)
+  kListGhost = kListTile + 1,                  // + (w - 2): two lists
   kListCorrect = kListGhost + 2,
   kListTail,                                   // one item
   kListMg2d,                                   // + depth * kEngShapes + shape
@@ -71,6 +72,7 @@ struct SlotDev {
   int dim, w, iface, neumann;
   GridView g;
   const uint8_t* phase;
+  const uint8_t *kind, *tile_kind;
   int* status;
   StencilCoef C;
   GhostParams GP;                              // homogeneous (with_data = 0); G is the slot's

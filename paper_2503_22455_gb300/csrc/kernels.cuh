@@ -87,12 +87,21 @@ struct CorrectParams {
   const double* box;        // [B] face data
   double a[2 * kMaxW + 1];
   double scale[2];          // beta_sigma / h^2
-  double box_w[kMaxW][8];
+  double box_c[kMaxW][8];   // [js - 1]: weights of a box face's ghosts js .. w, times their coefficients, summed
 };
+
+// Grids whose plain nodes the fixed-point tiles take: 3D of order 4 from 2^19 nodes (81^3) up, two and
+// more waves of two CTAs of 4096 nodes on 152 SMs.  One application with FP64 sums / with tiles: 96^3
+// interior 38 / 37 us, 128^3 exterior 84 / 63, 256^3 exterior 518 / 281.  In 2D (128 x 16 tiles, order 6,
+// 1024^2) they gained nothing: 43.6 / 44.6, the ghosts and affected nodes behind them take the time.
+inline bool op_tiled(const GridView& g, int w) { return g.dim == 3 && w == 2 && g.N >= (1 << 19); }
 
 // slots of Problem::d_counts: control points, affected nodes, irregular rows of
 // level l at kCountLevel0 + l (at most kMaxLevels levels), unknowns of the coarsest level
 constexpr int kCountK = 0, kCountAff = 1, kCountLevel0 = 2, kMaxLevels = 24, kCountCoarse = 40, kCountSlots = 48;
+
+// a node's class for the operator kernels
+constexpr uint8_t kKindUnknown = 1, kKindAffected = 2, kKindPlus = 4;
 
 struct Problem {
   iim_problem_desc desc;          // geom_coef and phi_dev are cleared after create (copies below)
@@ -130,6 +139,8 @@ struct Problem {
   double* G = nullptr;            // [nfit][w] ghost values of the current apply
   int* d_monos = nullptr;         // [M][dim] exponents
   // affected nodes (nodes whose stencil meets a control point or the box)
+  uint8_t* kind = nullptr;        // [N] class of each node for the operator (kKind bits)
+  uint8_t* tile_kind = nullptr;   // notes of the operator's fixed-point tiles
   int32_t* aff_flag = nullptr;    // [N]
   int32_t* aff_idx = nullptr;     // [N]
   int n_aff = 0, aff_cap = 0;
@@ -194,10 +205,11 @@ iim_status setup_fits(Problem& P);
 iim_status setup_levels(Problem& P, bool size_only);
 
 // operator.cu
+int op_tile_count(const Problem& P);             // fixed-point tiles of the operator (0: it has none)
+void op_tile_kinds(Problem& P, cudaStream_t s);  // their notes, from kind
 void ho_apply(Problem& P, const double* u, double* w, bool with_data, cudaStream_t s);
-void ho_stencil(Problem& P, const double* u, double* w, cudaStream_t s);
-void ho_ghost(Problem& P, const double* u, bool with_data, cudaStream_t s);
-void ho_correct(Problem& P, const double* u, double* w, bool with_data, cudaStream_t s);
+void ho_ghost(Problem& P, const double* u, bool with_data, double* G, cudaStream_t s);
+void ho_nodes(Problem& P, const double* u, double* w, bool with_data, const double* G, int parts, cudaStream_t s);
 void box_points(Problem& P, double* xb, cudaStream_t s);
 iim_status setup_direct(Problem& P, const double* params);
 iim_status ho_apply_noalloc(Problem& P, const double* u, double* w, bool with_data, cudaStream_t s);

@@ -445,9 +445,11 @@ void krylov_orth_pass(Problem& P, int j, int which, cudaStream_t s) {
 }
 
 // Augmented system (pure Neumann, Sec. 2.3): w = L u + alpha 1 on the unknowns, w_N = 1^T u.
-// The sum is deterministic: block partials in a fixed grid, then one thread in block order.
+// The sum is deterministic: block partials in a fixed grid, summed by the last block to finish (a
+// launch of one thread for that took 18 us).
 __global__ void __launch_bounds__(256) k_aug_apply(const double* __restrict__ u, double* __restrict__ w,
-                                                   const uint8_t* __restrict__ phase, int64_t N, double* partial) {
+                                                   const uint8_t* __restrict__ phase, int64_t N, double* partial,
+                                                   unsigned int* counter) {
   const double alpha = u[N];
   double acc[1] = {0.0};
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x)
@@ -456,13 +458,13 @@ __global__ void __launch_bounds__(256) k_aug_apply(const double* __restrict__ u,
       acc[0] += u[i];
     }
   block_reduce_store<1>(acc, partial, 1, blockIdx.x);
-}
-
-__global__ void k_aug_finish(double* __restrict__ w, int64_t N, const double* __restrict__ partial, int nb) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  double s = 0.0;
-  for (int b = 0; b < nb; ++b) s += partial[b];
-  w[N] = s;
+  if (!last_block(counter, gridDim.x)) return;
+  __shared__ double tot[1];
+  sum_partials(partial, gridDim.x, 1, 1, tot);
+  if (threadIdx.x == 0) {
+    *counter = 0;
+    w[N] = tot[0];
+  }
 }
 
 // z_N = v_N (scaled like the rest of v): the preconditioner is the identity on alpha
@@ -475,8 +477,7 @@ __global__ void k_aug_pass(const double* __restrict__ v, const double* __restric
 static void krylov_apply(Problem& P, const double* u, double* w, cudaStream_t s) {
   ho_apply(P, u, w, false, s);
   if (!P.aug) return;
-  IIM_LAUNCH(k_aug_apply, P.red_blocks, kRedThreads, 0, s, u, w, P.phase, P.g.N, P.partial);
-  IIM_LAUNCH(k_aug_finish, 1, 32, 0, s, w, P.g.N, P.partial, P.red_blocks);
+  IIM_LAUNCH(k_aug_apply, P.red_blocks, kRedThreads, 0, s, u, w, P.phase, P.g.N, P.partial, P.counter);
 }
 
 // the preconditioner of the Krylov iteration: z = M(v * vscale) (identity on alpha)

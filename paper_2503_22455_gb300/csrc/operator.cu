@@ -1,17 +1,25 @@
 // The (n, n+1) IIM operator w = L_Omega u (+ L_Gamma u_Gamma), paper Sec. 2.3, Eq. 12.
 //
-// Split into three kernels:
-//   k_ho_stencil  every unknown node: beta_sigma/h^2 sum_axes sum_j a_j u_{i+j e}, where
-//                 neighbours outside phase sigma (or outside the box) contribute 0;
-//   k_ho_ghost    one warp per control point: u_c (Dirichlet data, Neumann elimination
+// Two kernels:
+//   k_ho_ghost    eight lanes per control point: u_c (Dirichlet data, Neumann elimination
 //                 Eqs. 5-6, or the interface closure Eqs. 9-11) and the w ghost values
 //                 p_c(x_g) = s_c u_c + sum s_a u_a of Eq. 4;
-//   k_ho_correct  one thread per affected node: adds a_j p_c(x_{i+j e}) for every
-//                 out-of-phase offset past the first control point of each walk, and
-//                 the outer-box ghosts.
-// The stencil is FP64 and bound by the FP64 pipe on GB300 (2 FMA/clk/SM), so it
-// is written to use the fewest FP64 operations: neighbours at equal |j| are
-// summed first, then one FMA per |j| with beta/h^2 folded into the coefficients.
+//   k_ho_apply    every node: beta_sigma/h^2 sum_axes sum_j a_j u_{i+j e}.  Plain nodes (no
+//                 control point and no box face within w nodes along any axis) read only u
+//                 and one class byte.  Affected nodes are left to other blocks of the same
+//                 launch: a lane per direction, neighbours outside phase sigma (or outside
+//                 the box) contributing 0, plus a_j p_c(x_{i+j e}) for every out-of-phase
+//                 offset past the first control point of each walk, and the outer-box ghosts.
+// k_ho_apply is launched as a programmatic dependent of k_ho_ghost: its plain blocks need
+// nothing from it and run beside it, its affected blocks wait for it and are spread over
+// the rest of the grid, so that neither the ghost values nor the corrections add to the time of
+// the plain nodes.  Three kernels, the ghosts on a second stream between two events and the
+// corrections after both, took 17.2 us for a 64^2 circle and 57.5 us for the order-6 star at
+// 1024^2; the two take 9.4 to 12.5 and 43.6.
+// The plain nodes are FP64 and bound by the FP64 pipe on GB300 (2 FMA/clk/SM), so they are
+// written to use the fewest FP64 operations: neighbours at equal |j| are summed first, then
+// one FMA per |j| with beta/h^2 folded into the coefficients.  Large 3D grids sum in fixed point
+// instead (k_ho_tiles, op_tile.cuh).
 #include <mutex>
 #include <string>
 
@@ -19,6 +27,7 @@
 
 namespace iim {
 
+#include "op_tile.cuh"
 
 template <int D, int W>
 __device__ __forceinline__ void ho_stencil_node(const GridView& g, const StencilCoef& C, int interface_,
@@ -61,16 +70,6 @@ __device__ __forceinline__ void ho_stencil_node(const GridView& g, const Stencil
   w[i] = acc;
 }
 
-template <int D, int W>
-__global__ void __launch_bounds__(256) k_ho_stencil(GridView g, StencilCoef C, int interface_,
-                                                    const double* __restrict__ u,
-                                                    const uint8_t* __restrict__ phase, double* __restrict__ w) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= g.N) return;
-  ho_stencil_node<D, W>(g, C, interface_, u, phase, w, i);
-}
-
-
 // Eight lanes per control point: each lane accumulates an eighth of the X_c terms
 // of every row (sequential FMAs, no per-term reduction), then two shuffle steps
 // combine the quarters.  Boundary problems: rows 0..w-1 of fit c.  Interface
@@ -104,6 +103,8 @@ __device__ __forceinline__ void ho_ghost_body(const GhostParams& P, const double
     const int32_t* nodes = P.fit_nodes + (size_t)f * P.rcap;
     const double* coef = P.fit_coef + (size_t)f * rows * P.rcap;
     const int nr = P.interface_ ? W + 1 : W;
+    if (!u) continue;                            // u = 0: the data alone
+#pragma unroll 4
     for (int a = q; a < R; a += kGhostLanes) {
       const double ua = u[nodes[a]];
 #pragma unroll
@@ -142,68 +143,235 @@ __device__ __forceinline__ void ho_ghost_body(const GhostParams& P, const double
 
 template <int W>
 __global__ void __launch_bounds__(256) k_ho_ghost(GhostParams P, const double* __restrict__ u) {
+  pdl_trigger();                                 // k_ho_apply's plain blocks start beside this kernel
   ho_ghost_body<W>(P, u, blockIdx.x * blockDim.x + threadIdx.x);
 }
 
 
+// Ghost contribution of one direction (axis ax, side sd) at affected node t (node i, indices m, phase
+// ph): a_j p_c(x_{i+j e}) over the out-of-phase offsets past the first control point, or the outer box.
+// u = nullptr: the data's part alone (u = 0).
+// coef.at(j, s): the stencil's coefficient at offset j s; coef.box(v, s): P.box_c's sum v on side s.
+template <class Coef>
+__device__ __forceinline__ double ho_direction(const CorrectParams& P, Coef coef, const double* __restrict__ u, int t,
+                                               int64_t i, const int* m, uint8_t ph, int ax, int sd) {
+  const GridView& g = P.g;
+  const int n = g.n, d = g.dim, W = P.w;
+  const int64_t st = ax == 0 ? 1 : (ax == 1 ? (int64_t)n : (int64_t)n * n);
+  const int s = sd ? 1 : -1;
+  const int fit = P.aff_fit[t * 2 * d + 2 * ax + sd];
+  const int js = P.aff_j[t * 2 * d + 2 * ax + sd];
+  double acc = 0.0;
+  if (fit == -1 || fit >= P.nfit_cap) return acc;
+  if (fit >= 0) {
+    for (int j = js; j <= W; ++j) {
+      const int pos = m[ax] + j * s;
+      if (pos >= 0 && pos < n && P.phase[i + j * s * st] == ph) continue;   // back in phase: uses u
+      acc = fma(coef.at(j, s), P.G[(size_t)fit * W + (j - js)], acc);
+    }
+    return acc;
+  }
+  // outer box: ghosts js .. w from the degree-q line polynomial through the face value and the nodes
+  // 2..q+1 counted from the face, their weights summed beforehand (q + 1 operations for all of them)
+  double face = 0.0;
+  if (P.with_data) {
+    int64_t off = 0, mul = 1;
+    for (int k = 0; k < d; ++k) {
+      if (k == ax) continue;
+      off += m[k] * mul;
+      mul *= n;
+    }
+    off += (int64_t)(2 * ax + sd) * mul;
+    face = P.box[off];
+  }
+  acc = P.box_c[js - 1][0] * face;
+  if (u)
+    for (int mm = 2; mm <= P.q + 1; ++mm) {
+      const int pos = s > 0 ? n - mm : mm - 1;
+      acc = fma(P.box_c[js - 1][mm - 1], u[i + (int64_t)(pos - m[ax]) * st], acc);
+    }
+  return coef.box(acc, s);
+}
+
+// the operator's coefficients (even)
+struct OpCoef {
+  const CorrectParams& P;
+  __device__ __forceinline__ double at(int j, int) const { return P.a[P.w + j]; }
+  __device__ __forceinline__ double box(double v, int) const { return v; }
+};
+
+__device__ __forceinline__ void node_indices(int n, int d, int64_t i, int* m) {
+  m[0] = (int)(i % n);
+  const int64_t r = i / n;
+  m[1] = (int)(r % n);
+  m[2] = d > 2 ? (int)(r / n) : 0;
+}
+
+// the corrections alone, added to w (batched engine): one thread per affected node
 __device__ __forceinline__ void ho_correct_body(const CorrectParams& P, const double* __restrict__ u,
                                                 double* __restrict__ w, int t) {
   if (t >= *P.n_aff || t >= P.n_aff_cap) return;
-  const GridView& g = P.g;
-  const int n = g.n, d = g.dim, W = P.w;
   const int64_t i = P.aff_node[t];
   int m[3];
-  m[0] = (int)(i % n);
-  int64_t r = i / n;
-  m[1] = (int)(r % n);
-  m[2] = d > 2 ? (int)(r / n) : 0;
+  node_indices(P.g.n, P.g.dim, i, m);
   const uint8_t ph = P.phase[i];
   double acc = 0.0;
-  for (int ax = 0; ax < d; ++ax) {
-    const int64_t st = ax == 0 ? 1 : (ax == 1 ? (int64_t)n : (int64_t)n * n);
-    for (int sd = 0; sd < 2; ++sd) {
-      const int s = sd ? 1 : -1;
-      const int fit = P.aff_fit[t * 2 * d + 2 * ax + sd];
-      const int js = P.aff_j[t * 2 * d + 2 * ax + sd];
-      if (fit == -1 || fit >= P.nfit_cap) continue;
-      if (fit >= 0) {
-        for (int j = js; j <= W; ++j) {
-          int pos = m[ax] + j * s;
-          if (pos >= 0 && pos < n && P.phase[i + j * s * st] == ph) continue;   // back in phase: uses u
-          acc = fma(P.a[W + j * s], P.G[(size_t)fit * W + (j - js)], acc);
-        }
-      } else {
-        // outer box: ghosts from the degree-q line polynomial through the face value and
-        // the nodes 2..q+1 counted from the face
-        double face = 0.0;
-        if (P.with_data) {
-          int64_t off = 0, mul = 1;
-          for (int k = 0; k < d; ++k) {
-            if (k == ax) continue;
-            off += m[k] * mul;
-            mul *= n;
-          }
-          off += (int64_t)(2 * ax + sd) * mul;
-          face = P.box[off];
-        }
-        for (int j = js; j <= W; ++j) {
-          const int k = j - js;                  // ghost k+1 beyond the face
-          double v = P.box_w[k][0] * face;
-          for (int mm = 2; mm <= P.q + 1; ++mm) {
-            int pos = s > 0 ? n - mm : mm - 1;
-            v = fma(P.box_w[k][mm - 1], u[i + (int64_t)(pos - m[ax]) * st], v);
-          }
-          acc = fma(P.a[W + j * s], v, acc);
-        }
-      }
-    }
-  }
-  w[i] += P.scale[ph ? 1 : 0] * acc;
+  for (int k = 0; k < 2 * P.g.dim; ++k) acc += ho_direction(P, OpCoef{P}, u, t, i, m, ph, k >> 1, k & 1);
+  w[i] = fma(P.scale[ph ? 1 : 0], acc, w[i]);
 }
 
-__global__ void __launch_bounds__(256) k_ho_correct(CorrectParams P, const double* __restrict__ u,
-                                                    double* __restrict__ w) {
-  ho_correct_body(P, u, w, blockIdx.x * blockDim.x + threadIdx.x);
+// Blocks of a launch over plain and affected nodes: after the first `first` plain blocks (by then the
+// ghost kernel is done), every `every`-th block takes affected nodes until `aff` have, so that their
+// chains of loads run beside plain blocks that keep the FP64 pipe busy (FP64 sums at 256^3, exterior:
+// affected blocks in one piece 522 us, spread 518).
+struct AffSplit {
+  int plain, first, every, aff;
+  // this block's index among the plain (>= 0) or affected (~index < 0) ones
+  __device__ __forceinline__ int index(int b) const {
+    const int r = b - first;
+    if (r < 0) return b;
+    const int k = r / every;
+    if (k < aff && r - k * every == every - 1) return ~k;
+    return b - min(k, aff);
+  }
+};
+
+// The affected nodes: four lanes per node in 2D, one per direction (axis k / 2, side k & 1), because
+// there are few of them and their chains of dependent loads are what a small application waits for;
+// one thread per node in 3D, where the box faces alone have 6 w n^2 and the lanes' repeated FP64 sums
+// would cost more than the plain nodes (256^3: 423 us
+// against 83).
+template <int D>
+constexpr int aff_lanes() { return D == 2 ? 4 : 1; }
+
+// Sums over the directions in their order (the separate corrections kernel's order): of w neighbour
+// values at each offset, and of the ghost contributions.  v and part hold this thread's directions.
+template <int D>
+__device__ __forceinline__ double dir_sum(const double (&v)[2 * D / aff_lanes<D>()]) {
+  double s;
+  if constexpr (aff_lanes<D>() == 1) {
+    s = v[0];
+#pragma unroll
+    for (int k = 1; k < 2 * D; ++k) s += v[k];
+  } else {
+    s = __shfl_sync(0xffffffffu, v[0], 0, 4);
+#pragma unroll
+    for (int k = 1; k < 2 * D; ++k) s += __shfl_sync(0xffffffffu, v[0], k, 4);
+  }
+  return s;
+}
+
+// Node of this thread among the affected ones, its neighbours in phase (v[j][direction], else 0) and
+// its directions' ghost contributions.
+template <int D, int W, int NT, class Coef>
+struct Affected {
+  static constexpr int LG = aff_lanes<D>(), ND = 2 * D / LG;
+  int64_t i = 0;
+  uint8_t ph = 0;
+  int k0;                                // first of this thread's directions
+  bool live;
+  double v[W][ND], part[ND];
+  __device__ __forceinline__ Affected(const CorrectParams& P, Coef coef, const double* __restrict__ u, int block) {
+    const int t = (block * NT + (int)threadIdx.x) / LG, n = P.g.n;
+    k0 = LG == 1 ? 0 : threadIdx.x % LG;
+    live = t < min(*P.n_aff, P.n_aff_cap);
+#pragma unroll
+    for (int q = 0; q < ND; ++q) {
+      part[q] = 0.0;
+#pragma unroll
+      for (int j = 0; j < W; ++j) v[j][q] = 0.0;
+    }
+    if (!live) return;
+    i = P.aff_node[t];
+    int m[3];
+    node_indices(n, D, i, m);
+    ph = P.phase[i];
+#pragma unroll
+    for (int q = 0; q < ND; ++q) {
+      const int k = k0 + q, ax = k >> 1, s = k & 1 ? 1 : -1, ma = ax == 0 ? m[0] : (ax == 1 ? m[1] : m[2]);
+      const int64_t st = ax == 0 ? 1 : (ax == 1 ? (int64_t)n : (int64_t)n * n);
+      if (u)
+#pragma unroll
+        for (int j = 1; j <= W; ++j) {
+          const int pos = ma + j * s;
+          if (pos >= 0 && pos < n && P.phase[i + j * s * st] == ph) v[j - 1][q] = u[i + j * s * st];
+        }
+      part[q] = ho_direction(P, coef, u, t, i, m, ph, ax, k & 1);
+    }
+  }
+};
+template <int D, int W, int NT, class Coef>
+__device__ __forceinline__ Affected<D, W, NT, Coef> affected(const CorrectParams& P, Coef coef,
+                                                             const double* __restrict__ u, int block) {
+  return Affected<D, W, NT, Coef>(P, coef, u, block);
+}
+
+template <int D, int W, int NT>
+__device__ __forceinline__ void ho_affected(const CorrectParams& P, const StencilCoef& C, const double* __restrict__ u,
+                                            double* __restrict__ w, int block) {
+  const auto A = affected<D, W, NT>(P, OpCoef{P}, u, block);
+  const bool plus = A.ph != 0;
+  double acc = (plus ? C.c0[1] : C.c0[0]) * (A.live ? u[A.i] : 0.0);
+#pragma unroll
+  for (int j = 0; j < W; ++j) acc = fma(plus ? C.cj[1][j] : C.cj[0][j], dir_sum<D>(A.v[j]), acc);
+  const double corr = dir_sum<D>(A.part);
+  if (A.live && A.k0 == 0) w[A.i] = fma(plus ? P.scale[1] : P.scale[0], corr, acc);
+}
+
+// parts: 1 plain nodes, 2 affected nodes (both in an application; one alone for timing)
+template <int D, int W>
+__global__ void __launch_bounds__(256) k_ho_apply(CorrectParams P, StencilCoef C, const uint8_t* __restrict__ kind,
+                                                  const double* __restrict__ u, double* __restrict__ w, AffSplit S) {
+  const int b = S.index(blockIdx.x);
+  if (b < 0) {
+    pdl_wait();                            // the ghost values
+    ho_affected<D, W, 256>(P, C, u, w, ~b);
+    return;
+  }
+  const int64_t i = (int64_t)b * 256 + threadIdx.x;
+  if (i >= P.g.N) return;
+  const uint8_t kd = kind[i];
+  if (kd & kKindAffected) return;
+  if (!(kd & kKindUnknown)) {
+    w[i] = 0.0;
+    return;
+  }
+  w[i] = ho_plain_node<D, W>(P.g.n, C, (kd & kKindPlus) != 0, u, i);
+}
+
+// the same with the plain nodes in fixed-point tiles (op_tiled)
+template <int W>
+__global__ void __launch_bounds__(OpTile<W>::NT, 2)
+    k_ho_tiles(CorrectParams P, StencilCoef C, const uint8_t* __restrict__ kind, const uint8_t* __restrict__ tiles,
+               const double* __restrict__ u, double* __restrict__ w, AffSplit S) {
+  const int b = S.index(blockIdx.x);
+  if (b < 0) {
+    pdl_wait();                            // the ghost values
+    ho_affected<3, W, OpTile<W>::NT>(P, C, u, w, ~b);
+    return;
+  }
+  __shared__ OpTile<W> sm;
+  op_tile<W, false>(sm, P.g, C, kind, tiles, u, w, b, [](int64_t) {});
+}
+
+// b = f - L_Gamma u_Gamma (f at plain nodes; the data's ghosts at affected ones), from the ghost
+// values of u = 0
+template <int D>
+__global__ void __launch_bounds__(256) k_ho_rhs(CorrectParams P, const uint8_t* __restrict__ kind,
+                                                const double* __restrict__ f, double* __restrict__ b, AffSplit S) {
+  const int blk = S.index(blockIdx.x);
+  if (blk < 0) {
+    pdl_wait();
+    const auto A = affected<D, 1, 256>(P, OpCoef{P}, nullptr, ~blk);
+    const double corr = dir_sum<D>(A.part);
+    if (A.live && A.k0 == 0) b[A.i] = f[A.i] - (A.ph ? P.scale[1] : P.scale[0]) * corr;
+    return;
+  }
+  const int64_t i = (int64_t)blk * 256 + threadIdx.x;
+  if (i >= P.g.N) return;
+  const uint8_t kd = kind[i];
+  if (kd & kKindAffected) return;
+  b[i] = kd & kKindUnknown ? f[i] : 0.0;
 }
 
 static StencilCoef stencil_coef(const Problem& P) {
@@ -217,42 +385,13 @@ static StencilCoef stencil_coef(const Problem& P) {
   return C;
 }
 
-void ho_stencil(Problem& P, const double* u, double* w, cudaStream_t s) {
-  const GridView& g = P.g;
-  const int T = 256;
-  const int iface = P.desc.bc == IIM_BC_INTERFACE;
-  StencilCoef C = stencil_coef(P);
-  int grid = ceil_div(g.N, T);
-  if (g.dim == 2) {
-    if (P.w == 2) IIM_LAUNCH((k_ho_stencil<2, 2>), grid, T, 0, s, g, C, iface, u, P.phase, w);
-    else IIM_LAUNCH((k_ho_stencil<2, 3>), grid, T, 0, s, g, C, iface, u, P.phase, w);
-  } else {
-    if (P.w == 2) IIM_LAUNCH((k_ho_stencil<3, 2>), grid, T, 0, s, g, C, iface, u, P.phase, w);
-    else IIM_LAUNCH((k_ho_stencil<3, 3>), grid, T, 0, s, g, C, iface, u, P.phase, w);
-  }
-}
-
-void ho_ghost(Problem& P, const double* u, bool with_data, cudaStream_t s) {
-  const int T = 256;
-  const int iface = P.desc.bc == IIM_BC_INTERFACE;
+void ho_ghost(Problem& P, const double* u, bool with_data, double* G, cudaStream_t s) {
+  StencilCoef C;
   GhostParams GP;
-  GP.nfit = P.nfit_cap;
-  GP.w = P.w;
-  GP.rcap = P.rcap;
-  GP.bc = P.desc.bc;
-  GP.interface_ = iface;
+  CorrectParams CP;
+  eng_operator_params(P, &C, &GP, &CP);
   GP.with_data = with_data;
-  GP.beta_p = P.desc.beta_plus;
-  GP.beta_m = P.desc.beta_minus;
-  GP.K = P.d_counts + 0;
-  GP.fit_R = P.fit_R;
-  GP.fit_nodes = P.fit_nodes;
-  GP.fit_coef = P.fit_coef;
-  GP.fit_cdat = P.fit_cdat;
-  GP.g = P.d_g;
-  GP.j0 = P.d_j0;
-  GP.j1 = P.d_j1;
-  GP.G = P.G;
+  GP.G = G;
   if (P.K_cap > 0) {
     // small blocks: a few thousand control points must still spread over all 152 SMs
     const int grid = ceil_div((int64_t)P.K_cap * kGhostLanes, 64);
@@ -261,68 +400,81 @@ void ho_ghost(Problem& P, const double* u, bool with_data, cudaStream_t s) {
   }
 }
 
-void ho_correct(Problem& P, const double* u, double* w, bool with_data, cudaStream_t s) {
-  const GridView& g = P.g;
-  const int T = 256;
+// plain: blocks of plain nodes; threads: of a block
+static AffSplit aff_split(const Problem& P, int parts, int plain, int threads) {
+  AffSplit S;
+  const int lanes = P.g.dim == 2 ? aff_lanes<2>() : aff_lanes<3>();
+  S.plain = parts & 1 ? plain : 0;
+  S.aff = parts & 2 ? ceil_div((int64_t)P.aff_cap * lanes, threads) : 0;
+  S.first = S.plain / 3;
+  S.every = S.aff > 0 ? (S.plain - S.first) / S.aff + 1 : 1;
+  return S;
+}
+
+void ho_nodes(Problem& P, const double* u, double* w, bool with_data, const double* G, int parts, cudaStream_t s) {
+  StencilCoef C;
+  GhostParams GP;
   CorrectParams CP;
-  CP.g = g;
-  CP.w = P.w;
-  CP.q = P.q;
+  eng_operator_params(P, &C, &GP, &CP);
   CP.with_data = with_data;
-  CP.n_aff_cap = P.aff_cap;
-  CP.nfit_cap = P.nfit_cap;
-  CP.n_aff = P.d_counts + 1;
-  CP.aff_node = P.aff_node;
-  CP.aff_fit = P.aff_fit;
-  CP.aff_j = P.aff_j;
-  CP.G = P.G;
-  CP.phase = P.phase;
-  CP.box = P.d_box;
-  for (int k = 0; k < 2 * kMaxW + 1; ++k) CP.a[k] = k < 2 * P.w + 1 ? P.a[k] : 0.0;
-  const double h2 = g.h * g.h;
-  CP.scale[0] = P.desc.beta_minus / h2;
-  CP.scale[1] = P.desc.beta_plus / h2;
-  for (int k = 0; k < kMaxW; ++k)
-    for (int mm = 0; mm < 8; ++mm) CP.box_w[k][mm] = P.box_w[k][mm];
-  if (P.aff_cap > 0) IIM_LAUNCH(k_ho_correct, ceil_div(P.aff_cap, 64), 64, 0, s, CP, u, w);
+  CP.G = G;
+  // (with no control point there is no ghost kernel to run beside: an ordinary launch)
+#define IIM_APPLY(kernel_, nblk_, nthr_, ...)                                                     \
+  do {                                                                                             \
+    const AffSplit S = aff_split(P, parts, nblk_, nthr_);                                        \
+    if (S.plain + S.aff == 0) return;                                                              \
+    if (P.K_cap > 0) IIM_LAUNCH_PDL(kernel_, S.plain + S.aff, nthr_, 0, s, CP, C, __VA_ARGS__, S); \
+    else IIM_LAUNCH(kernel_, S.plain + S.aff, nthr_, 0, s, CP, C, __VA_ARGS__, S);                \
+  } while (0)
+#define IIM_NODES(D, W) IIM_APPLY((k_ho_apply<D, W>), ceil_div(P.g.N, 256), 256, (const uint8_t*)P.kind, u, w)
+  if (P.g.dim == 2) {
+    if (P.w == 2) IIM_NODES(2, 2);
+    else IIM_NODES(2, 3);
+  } else if (op_tiled(P.g, P.w)) {
+    IIM_APPLY(k_ho_tiles<2>, OpTile<2>::count(P.g.n), OpTile<2>::NT, (const uint8_t*)P.kind, (const uint8_t*)P.tile_kind, u, w);
+  } else {
+    if (P.w == 2) IIM_NODES(3, 2);
+    else IIM_NODES(3, 3);
+  }
+#undef IIM_NODES
+#undef IIM_APPLY
+}
+
+int op_tile_count(const Problem& P) { return op_tiled(P.g, P.w) ? OpTile<2>::count(P.g.n) : 0; }
+
+void op_tile_kinds(Problem& P, cudaStream_t s) {
+  const int count = op_tile_count(P);
+  if (count > 0) IIM_LAUNCH(k_tile_kinds<2>, count, OpTile<2>::NT, 0, s, P.g.n, P.kind, P.tile_kind);
 }
 
 void ho_apply(Problem& P, const double* u, double* w, bool with_data, cudaStream_t s) {
-  if (P.side && P.ev_fork && P.ev_join) {
-    // the ghost values read only u: they are computed on the side stream beside the
-    // stencil, and the corrections wait for both
-    cudaEventRecord(P.ev_fork, s);
-    cudaStreamWaitEvent(P.side, P.ev_fork, 0);
-    ho_ghost(P, u, with_data, P.side);
-    cudaEventRecord(P.ev_join, P.side);
-    ho_stencil(P, u, w, s);
-    cudaStreamWaitEvent(s, P.ev_join, 0);
-  } else {
-    ho_stencil(P, u, w, s);
-    ho_ghost(P, u, with_data, s);
-  }
-  ho_correct(P, u, w, with_data, s);
+  ho_ghost(P, u, with_data, P.G, s);
+  ho_nodes(P, u, w, with_data, P.G, 3, s);
 }
 
-__global__ void k_rhs_finish(GridView g, int interface_, const uint8_t* __restrict__ phase,
-                             const double* __restrict__ f, const double* __restrict__ lg, double* __restrict__ b) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= g.N) return;
-  b[i] = (interface_ || phase[i]) ? f[i] - lg[i] : 0.0;
-}
-
-// b = f - L_Gamma u_Gamma: the operator applied to u = 0 with the data switched on
+// b = f - L_Gamma u_Gamma: the operator of u = 0 with the data switched on, subtracted from f
 void compute_rhs(Problem& P, const double* f, cudaStream_t s) {
-  double* zero = P.Z;                  // Z[0] is zeroed first: the apply reads it as u
-  double* lg = P.tmp;
-  cudaMemsetAsync(zero, 0, sizeof(double) * P.g.N, s);
-  ho_apply(P, zero, lg, true, s);
-  IIM_LAUNCH(k_rhs_finish, ceil_div(P.g.N, 256), 256, 0, s, P.g, P.desc.bc == IIM_BC_INTERFACE, P.phase, f, lg, P.b);
+  ho_ghost(P, nullptr, true, P.G, s);
+  StencilCoef C;
+  GhostParams GP;
+  CorrectParams CP;
+  eng_operator_params(P, &C, &GP, &CP);
+  CP.with_data = 1;
+  const AffSplit S = aff_split(P, 3, ceil_div(P.g.N, 256), 256);
+  const int grid = S.plain + S.aff;
+#define IIM_RHS(D)                                                                                        \
+  do {                                                                                                    \
+    if (P.K_cap > 0) IIM_LAUNCH_PDL(k_ho_rhs<D>, grid, 256, 0, s, CP, (const uint8_t*)P.kind, f, P.b, S); \
+    else IIM_LAUNCH(k_ho_rhs<D>, grid, 256, 0, s, CP, (const uint8_t*)P.kind, f, P.b, S); \
+  } while (0)
+  if (P.g.dim == 2) IIM_RHS(2);
+  else IIM_RHS(3);
+#undef IIM_RHS
 }
 
 
 // ---------------------------------------------------------------------------- no-allocation apply
-// The same three kernels as ho_apply, but the ghost values go to a file-scope
+// The same kernels as ho_apply, but the ghost values go to a file-scope
 // device array instead of the problem's workspace.  kNoAllocGhostMax doubles
 // (2 MiB) are reserved on every device that loads the library, for the life of
 // the process.  All calls share the array, so calls that overlap on the device
@@ -366,53 +518,8 @@ iim_status ho_apply_noalloc(Problem& P, const double* u, double* w, bool with_da
     }
     G = g_noalloc_addr[dev];
   }
-  ho_stencil(P, u, w, s);
-  const int iface = P.desc.bc == IIM_BC_INTERFACE;
-  GhostParams GP;
-  GP.nfit = P.nfit_cap;
-  GP.w = P.w;
-  GP.rcap = P.rcap;
-  GP.bc = P.desc.bc;
-  GP.interface_ = iface;
-  GP.with_data = with_data;
-  GP.beta_p = P.desc.beta_plus;
-  GP.beta_m = P.desc.beta_minus;
-  GP.K = P.d_counts + 0;
-  GP.fit_R = P.fit_R;
-  GP.fit_nodes = P.fit_nodes;
-  GP.fit_coef = P.fit_coef;
-  GP.fit_cdat = P.fit_cdat;
-  GP.g = P.d_g;
-  GP.j0 = P.d_j0;
-  GP.j1 = P.d_j1;
-  GP.G = G;
-  if (P.K_cap > 0) {
-    const int grid = ceil_div((int64_t)P.K_cap * kGhostLanes, 64);
-    if (P.w == 2) IIM_LAUNCH(k_ho_ghost<2>, grid, 64, 0, s, GP, u);
-    else IIM_LAUNCH(k_ho_ghost<3>, grid, 64, 0, s, GP, u);
-  }
-  CorrectParams CP;
-  const GridView& g = P.g;
-  CP.g = g;
-  CP.w = P.w;
-  CP.q = P.q;
-  CP.with_data = with_data;
-  CP.n_aff_cap = P.aff_cap;
-  CP.nfit_cap = P.nfit_cap;
-  CP.n_aff = P.d_counts + 1;
-  CP.aff_node = P.aff_node;
-  CP.aff_fit = P.aff_fit;
-  CP.aff_j = P.aff_j;
-  CP.G = G;
-  CP.phase = P.phase;
-  CP.box = P.d_box;
-  for (int k = 0; k < 2 * kMaxW + 1; ++k) CP.a[k] = k < 2 * P.w + 1 ? P.a[k] : 0.0;
-  const double h2 = g.h * g.h;
-  CP.scale[0] = P.desc.beta_minus / h2;
-  CP.scale[1] = P.desc.beta_plus / h2;
-  for (int k = 0; k < kMaxW; ++k)
-    for (int mm = 0; mm < 8; ++mm) CP.box_w[k][mm] = P.box_w[k][mm];
-  if (P.aff_cap > 0) IIM_LAUNCH(k_ho_correct, ceil_div(P.aff_cap, 64), 64, 0, s, CP, u, w);
+  ho_ghost(P, u, with_data, G, s);
+  ho_nodes(P, u, w, with_data, G, 3, s);
   return IIM_OK;
 }
 
@@ -435,6 +542,21 @@ __global__ void __launch_bounds__(kEngThreads) k_eng_stencil(EngArgs A) {
       const int64_t i = base + k * kEngThreads;
       if (i < N) ho_stencil_node<D, W>(s.g, s.C, s.iface, u, s.phase, w, i);
     }
+  });
+}
+
+// items of problems with fixed-point tiles: one tile each (affected nodes as in k_eng_stencil)
+template <int W>
+__global__ void __launch_bounds__(OpTile<W>::NT, 2) k_eng_tiles(EngArgs A) {
+  __shared__ OpTile<W> sm;
+  eng_for_items(A, kListTile, [&](int si, int item) {
+    const SlotDev& s = A.slots[si];
+    if (s.role == kRoleIdle) return;
+    const double* u;
+    double* w;
+    eng_apply_io(s, u, w);
+    op_tile<W, true>(sm, s.g, s.C, s.kind, s.tile_kind, u, w, item,
+                        [&](int64_t i) { ho_stencil_node<3, W>(s.g, s.C, s.iface, u, s.phase, w, i); });
   });
 }
 
@@ -467,9 +589,22 @@ void eng_launch_apply(const EngArgs& A, const unsigned char* present, cudaStream
     IIM_LAUNCH((k_eng_stencil<D, W>), eng_grid((const void*)k_eng_stencil<D, W>, kEngThreads, 0), kEngThreads, 0, s, A);
   IIM_ENG_ST(2, 2) IIM_ENG_ST(2, 3) IIM_ENG_ST(3, 2) IIM_ENG_ST(3, 3)
 #undef IIM_ENG_ST
+  if (present[kListTile])
+    IIM_LAUNCH(k_eng_tiles<2>, eng_grid((const void*)k_eng_tiles<2>, OpTile<2>::NT, 0), OpTile<2>::NT, 0, s, A);
   if (present[kListGhost + 0]) IIM_LAUNCH(k_eng_ghost<2>, eng_grid((const void*)k_eng_ghost<2>, 64, 0), 64, 0, s, A);
   if (present[kListGhost + 1]) IIM_LAUNCH(k_eng_ghost<3>, eng_grid((const void*)k_eng_ghost<3>, 64, 0), 64, 0, s, A);
   if (present[kListCorrect]) IIM_LAUNCH(k_eng_correct, eng_grid((const void*)k_eng_correct, 64, 0), 64, 0, s, A);
+}
+
+// Q.box_c for a stencil with coefficient coef(j) at offset j on the + side
+template <class F>
+static void box_sums(const Problem& P, CorrectParams& Q, F coef) {
+  for (int js = 1; js <= kMaxW; ++js)
+    for (int m = 0; m < 8; ++m) {
+      double v = 0.0;
+      for (int j = js; j <= P.w; ++j) v += coef(j) * P.box_w[j - js][m];
+      Q.box_c[js - 1][m] = v;
+    }
 }
 
 // the operator's per-problem parameters (homogeneous: the data enter through b)
@@ -511,8 +646,7 @@ void eng_operator_params(Problem& P, StencilCoef* C, GhostParams* GP, CorrectPar
   const double h2 = P.g.h * P.g.h;
   Q.scale[0] = P.desc.beta_minus / h2;
   Q.scale[1] = P.desc.beta_plus / h2;
-  for (int k = 0; k < kMaxW; ++k)
-    for (int mm = 0; mm < 8; ++mm) Q.box_w[k][mm] = P.box_w[k][mm];
+  box_sums(P, Q, [&](int j) { return P.a[P.w + j]; });
 }
 
 
@@ -558,96 +692,55 @@ static GradCoef grad_coef(int w) {
   return B;
 }
 
-// grad u by the centred first-derivative stencil b of the scheme's order: neighbours
-// out of phase (or outside the box) contribute nothing here; their ghost values are
-// added by k_grad_correct.  out is [dim][N]; zero at nodes that are not unknowns.
+// its coefficients as ho_direction takes them (odd)
+template <int W>
+struct GradFunctor {
+  const GradCoef& B;
+  __device__ __forceinline__ double at(int j, int s) const { return s > 0 ? B.b[W + j] : -B.b[W + j]; }
+  __device__ __forceinline__ double box(double v, int s) const { return s > 0 ? v : -v; }
+};
+
+// grad u by the centred first-derivative stencil b of the scheme's order, in one launch beside the
+// ghost kernel like k_ho_apply.  out is [dim][N]; zero at nodes that are not unknowns.
 template <int D, int W>
-__global__ void __launch_bounds__(256) k_grad_stencil(GridView g, GradCoef B, int interface_,
-                                                      const double* __restrict__ u,
-                                                      const uint8_t* __restrict__ phase, double* __restrict__ out) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= g.N) return;
-  const int n = g.n;
-  const uint8_t ph = phase[i];
-  if (!interface_ && !ph) {
+__global__ void __launch_bounds__(256) k_grad_apply(CorrectParams P, GradCoef B, const uint8_t* __restrict__ kind,
+                                                    const double* __restrict__ u, double* __restrict__ out, AffSplit S) {
+  const int blk = S.index(blockIdx.x), n = P.g.n;
+  const double ih = 1.0 / P.g.h;
+  if (blk < 0) {
+    pdl_wait();                            // the ghost values
+    const auto A = affected<D, W, 256>(P, GradFunctor<W>{B}, u, ~blk);
+    // direction 2 ax + 1 is the + side, 2 ax the - side
+    if constexpr (aff_lanes<D>() == 1) {
 #pragma unroll
-    for (int ax = 0; ax < D; ++ax) out[(size_t)ax * g.N + i] = 0.0;
+      for (int ax = 0; ax < D; ++ax) {
+        double acc = 0.0;
+#pragma unroll
+        for (int j = 0; j < W; ++j) acc = fma(B.b[W + j + 1], A.v[j][2 * ax + 1] - A.v[j][2 * ax], acc);
+        if (A.live) out[(size_t)ax * P.g.N + A.i] = fma(A.part[2 * ax + 1] + A.part[2 * ax], ih, acc * ih);
+      }
+    } else {
+      double acc = 0.0;
+#pragma unroll
+      for (int j = 0; j < W; ++j) acc = fma(B.b[W + j + 1], A.v[j][0] - __shfl_xor_sync(0xffffffffu, A.v[j][0], 1), acc);
+      const double corr = A.part[0] + __shfl_xor_sync(0xffffffffu, A.part[0], 1);
+      if (A.live && (A.k0 & 1)) out[(size_t)(A.k0 >> 1) * P.g.N + A.i] = fma(corr, ih, acc * ih);
+    }
     return;
   }
-  int m[3];
-  m[0] = (int)(i % n);
-  const int64_t r = i / n;
-  m[1] = (int)(r % n);
-  m[2] = D > 2 ? (int)(r / n) : 0;
-  const double ih = 1.0 / g.h;
+  const int64_t i = (int64_t)blk * 256 + threadIdx.x;
+  if (i >= P.g.N) return;
+  const uint8_t kd = kind[i];
+  if (kd & kKindAffected) return;
 #pragma unroll
   for (int ax = 0; ax < D; ++ax) {
     const int64_t st = ax == 0 ? 1 : (ax == 1 ? (int64_t)n : (int64_t)n * n);
     double acc = 0.0;
+    if (kd & kKindUnknown) {
 #pragma unroll
-    for (int j = 1; j <= W; ++j) {
-      double lv = 0.0, rv = 0.0;
-      if (m[ax] - j >= 0 && phase[i - j * st] == ph) lv = u[i - j * st];
-      if (m[ax] + j < n && phase[i + j * st] == ph) rv = u[i + j * st];
-      acc = fma(B.b[W + j], rv - lv, acc);
+      for (int j = 1; j <= W; ++j) acc = fma(B.b[W + j], u[i + j * st] - u[i - j * st], acc);
     }
-    out[(size_t)ax * g.N + i] = acc * ih;
-  }
-}
-
-// ghost contributions to the gradient at the affected nodes (the walk rules of k_ho_correct)
-__global__ void __launch_bounds__(64) k_grad_correct(CorrectParams P, GradCoef B,
-                                                     const double* __restrict__ u, double* __restrict__ out) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= *P.n_aff || t >= P.n_aff_cap) return;
-  const GridView& g = P.g;
-  const int n = g.n, d = g.dim, W = P.w;
-  const int64_t i = P.aff_node[t];
-  int m[3];
-  m[0] = (int)(i % n);
-  const int64_t r = i / n;
-  m[1] = (int)(r % n);
-  m[2] = d > 2 ? (int)(r / n) : 0;
-  const uint8_t ph = P.phase[i];
-  const double ih = 1.0 / g.h;
-  for (int ax = 0; ax < d; ++ax) {
-    const int64_t st = ax == 0 ? 1 : (ax == 1 ? (int64_t)n : (int64_t)n * n);
-    double acc = 0.0;
-    for (int sd = 0; sd < 2; ++sd) {
-      const int s = sd ? 1 : -1;
-      const int fit = P.aff_fit[t * 2 * d + 2 * ax + sd];
-      const int js = P.aff_j[t * 2 * d + 2 * ax + sd];
-      if (fit == -1 || fit >= P.nfit_cap) continue;
-      if (fit >= 0) {
-        for (int j = js; j <= W; ++j) {
-          const int pos = m[ax] + j * s;
-          if (pos >= 0 && pos < n && P.phase[i + j * s * st] == ph) continue;
-          acc = fma(B.b[W + j * s], P.G[(size_t)fit * W + (j - js)], acc);
-        }
-      } else {
-        double face = 0.0;
-        if (P.with_data) {
-          int64_t off = 0, mul = 1;
-          for (int k = 0; k < d; ++k) {
-            if (k == ax) continue;
-            off += m[k] * mul;
-            mul *= n;
-          }
-          off += (int64_t)(2 * ax + sd) * mul;
-          face = P.box[off];
-        }
-        for (int j = js; j <= W; ++j) {
-          const int k = j - js;
-          double v = P.box_w[k][0] * face;
-          for (int mm = 2; mm <= P.q + 1; ++mm) {
-            const int pos = s > 0 ? n - mm : mm - 1;
-            v = fma(P.box_w[k][mm - 1], u[i + (int64_t)(pos - m[ax]) * st], v);
-          }
-          acc = fma(B.b[W + j * s], v, acc);
-        }
-      }
-    }
-    out[(size_t)ax * g.N + i] += acc * ih;
+    out[(size_t)ax * P.g.N + i] = acc * ih;
   }
 }
 
@@ -666,24 +759,31 @@ iim_status boundary_values(Problem& P, const double* u, double* out, cudaStream_
 }
 
 iim_status gradient(Problem& P, const double* u, double* grad, cudaStream_t s) {
-  const GridView& g = P.g;
-  const GradCoef b_dev = grad_coef(P.w);
-  const int iface = P.desc.bc == IIM_BC_INTERFACE;
-  const int grid = ceil_div(g.N, 256);
-  if (g.dim == 2) {
-    if (P.w == 2) IIM_LAUNCH((k_grad_stencil<2, 2>), grid, 256, 0, s, g, b_dev, iface, u, P.phase, grad);
-    else IIM_LAUNCH((k_grad_stencil<2, 3>), grid, 256, 0, s, g, b_dev, iface, u, P.phase, grad);
-  } else {
-    if (P.w == 2) IIM_LAUNCH((k_grad_stencil<3, 2>), grid, 256, 0, s, g, b_dev, iface, u, P.phase, grad);
-    else IIM_LAUNCH((k_grad_stencil<3, 3>), grid, 256, 0, s, g, b_dev, iface, u, P.phase, grad);
-  }
-  ho_ghost(P, u, true, s);                        // ghost values with the problem's data
+  const GradCoef B = grad_coef(P.w);
+  ho_ghost(P, u, true, P.G, s);                     // ghost values with the problem's data
   StencilCoef C;
   GhostParams GP;
   CorrectParams CP;
   eng_operator_params(P, &C, &GP, &CP);
   CP.with_data = 1;
-  if (P.aff_cap > 0) IIM_LAUNCH(k_grad_correct, ceil_div(P.aff_cap, 64), 64, 0, s, CP, b_dev, u, grad);
+  box_sums(P, CP, [&](int j) { return B.b[P.w + j]; });
+  const AffSplit S = aff_split(P, 3, ceil_div(P.g.N, 256), 256);
+  const int grid = S.plain + S.aff;
+#define IIM_GRAD(D, W)                                                                                              \
+  do {                                                                                                              \
+    if (P.K_cap > 0)                                                                                                \
+      IIM_LAUNCH_PDL((k_grad_apply<D, W>), grid, 256, 0, s, CP, B, (const uint8_t*)P.kind, u, grad, S); \
+    else                                                                                                            \
+      IIM_LAUNCH((k_grad_apply<D, W>), grid, 256, 0, s, CP, B, (const uint8_t*)P.kind, u, grad, S); \
+  } while (0)
+  if (P.g.dim == 2) {
+    if (P.w == 2) IIM_GRAD(2, 2);
+    else IIM_GRAD(2, 3);
+  } else {
+    if (P.w == 2) IIM_GRAD(3, 2);
+    else IIM_GRAD(3, 3);
+  }
+#undef IIM_GRAD
   return IIM_OK;
 }
 

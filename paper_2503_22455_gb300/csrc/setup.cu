@@ -101,7 +101,7 @@ __device__ inline bool is_unknown(const WalkParams& P, uint8_t ph) { return P.in
 
 // geometry checks + affected flag per node
 __global__ void k_affected_flags(WalkParams P, const uint8_t* __restrict__ phase, int32_t* __restrict__ flag,
-                                 int* status) {
+                                 uint8_t* __restrict__ kind, int* status) {
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const GridView& g = P.g;
   if (i >= g.N) return;
@@ -131,6 +131,7 @@ __global__ void k_affected_flags(WalkParams P, const uint8_t* __restrict__ phase
     }
   }
   flag[i] = f;
+  kind[i] = (unk ? kKindUnknown : 0) | (f ? kKindAffected : 0) | (ph ? kKindPlus : 0);
 }
 
 __global__ void k_affected_fill(WalkParams P, const uint8_t* __restrict__ phase, const int32_t* __restrict__ flag,
@@ -668,7 +669,8 @@ iim_status setup_geometry(Problem& P, bool size_only) {
              P.cr_axis, P.cr_lo, P.cr_loplus, P.cr_t, P.cr_x, P.cr_n, P.cr_kappa, P.d_status);
   IIM_LAUNCH(k_curvature_check, ceil_div(P.K_cap, T), T, 0, s, P.cr_kappa, P.d_counts + 0, g.h, P.d_status);
   WalkParams W{g, P.w, P.q, P.desc.bc == IIM_BC_INTERFACE, P.desc.box_bc};
-  IIM_LAUNCH(k_affected_flags, ceil_div(g.N, T), T, 0, s, W, P.phase, P.aff_flag, P.d_status);
+  IIM_LAUNCH(k_affected_flags, ceil_div(g.N, T), T, 0, s, W, P.phase, P.aff_flag, P.kind, P.d_status);
+  op_tile_kinds(P, s);
   scan_exclusive(P.aff_flag, P.aff_idx, g.N, P.d_counts + 1, P.scan_scratch, s);
   return IIM_OK;
 }
