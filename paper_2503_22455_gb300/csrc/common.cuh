@@ -432,6 +432,41 @@ __device__ inline double warp_sum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
+// Sums of the N values of every lane over groups of LANES lanes (hl: lane in the group), to
+// out[0 .. N).  Groups of P
+// values are transposed: P - 1 additions leave each lane with part of one sum, where a butterfly per
+// value takes 5 each; FP64 additions hold a scheduler for 64 clocks.  Every sum is the tree of the
+// butterfly (lanes 16 apart first), so it has the same bits.
+template <int LANES, int N>
+__device__ __forceinline__ void lane_sums(double* v, int hl, double* out) {
+  if constexpr (N > 0) {
+    constexpr int P0 = N >= 32 ? 32 : N >= 16 ? 16 : N >= 8 ? 8 : N >= 4 ? 4 : N >= 2 ? 2 : 1;
+    // a group that is more than five eighths full is cheaper padded than split
+    constexpr int P1 = N < 32 && P0 != N && 8 * N > 10 * P0 ? 2 * P0 : P0;
+    constexpr int P = P1 < LANES ? P1 : LANES;
+    constexpr int TAKE = N < P ? N : P;
+    double w[P];
+#pragma unroll
+    for (int i = 0; i < P; ++i) w[i] = i < TAKE ? v[i] : 0.0;
+    int o = LANES / 2;
+#pragma unroll
+    for (int n = P; n > 1; n >>= 1, o >>= 1) {
+      const bool hi = (hl & o) != 0;
+#pragma unroll
+      for (int i = 0; i < n / 2; ++i) {
+        const double mine = hi ? w[i + n / 2] : w[i], other = hi ? w[i] : w[i + n / 2];
+        w[i] = mine + __shfl_xor_sync(0xffffffffu, other, o);
+      }
+    }
+    double r = w[0];
+#pragma unroll
+    for (int k = LANES / P / 2; k > 0; k >>= 1) r += __shfl_xor_sync(0xffffffffu, r, k);
+    const int mine = hl / (LANES / P);
+    if (hl % (LANES / P) == 0 && mine < TAKE) out[mine] = r;
+    lane_sums<LANES, N - TAKE>(v + TAKE, hl, out + TAKE);
+  }
+}
+
 __device__ inline float warp_sumf(float v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;

@@ -48,19 +48,18 @@ enum EngList {
 };
 
 // Per-tick lists: the plan kernel copies every static list above, keeping only the
-// slots whose role this tick uses it, plus three lists that select by role alone.
-enum EngDynList { kDynAllIter = kListCount, kDynAllRestart, kDynRedRestart, kDynCount };
+// slots whose role this tick uses it, plus one that selects by role alone.
+enum EngDynList { kDynRedRestart = kListCount, kDynCount };
 constexpr int kMaskIter = 1 << kRoleIter, kMaskRestart = 1 << kRoleRestart;
 
 // roles that use dynamic list k
 __host__ __device__ inline int eng_list_mask(int k) {
-  if (k == kListXup || k == kDynAllRestart || k == kDynRedRestart) return kMaskRestart;
+  if (k == kListXup || k == kDynRedRestart) return kMaskRestart;
   if (k == kListAll || (k >= kListStencil && k <= kListCorrect)) return kMaskIter | kMaskRestart;
   return kMaskIter;                            // reductions of the iteration, Arnoldi, the V-cycle
 }
 // the static list a dynamic list is drawn from
 __host__ __device__ inline int eng_list_source(int k) {
-  if (k == kDynAllIter || k == kDynAllRestart) return kListAll;
   if (k == kDynRedRestart) return kListRed;
   return k;
 }

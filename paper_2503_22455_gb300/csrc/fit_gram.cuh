@@ -106,38 +106,6 @@ struct GramSmem {                        // one fit
   int code[S::ROWS];                     // window position of each row's node, i0 | i1 << 5 | i2 << 10
 };
 
-// Sums of the N values of every lane over the LANES lanes of a fit, to out[0 .. N).  Groups of P
-// values are transposed: P - 1 additions leave each lane with part of one sum.
-template <int LANES, int N>
-__device__ __forceinline__ void gram_reduce(double* v, int hl, double* out) {
-  if constexpr (N > 0) {
-    constexpr int P0 = N >= 32 ? 32 : N >= 16 ? 16 : N >= 8 ? 8 : N >= 4 ? 4 : N >= 2 ? 2 : 1;
-    // a group that is more than five eighths full is cheaper padded than split
-    constexpr int P1 = N < 32 && P0 != N && 8 * N > 10 * P0 ? 2 * P0 : P0;
-    constexpr int P = P1 < LANES ? P1 : LANES;
-    constexpr int TAKE = N < P ? N : P;
-    double w[P];
-#pragma unroll
-    for (int i = 0; i < P; ++i) w[i] = i < TAKE ? v[i] : 0.0;
-    int o = LANES / 2;
-#pragma unroll
-    for (int n = P; n > 1; n >>= 1, o >>= 1) {
-      const bool hi = (hl & o) != 0;
-#pragma unroll
-      for (int i = 0; i < n / 2; ++i) {
-        const double mine = hi ? w[i + n / 2] : w[i], other = hi ? w[i] : w[i + n / 2];
-        w[i] = mine + __shfl_xor_sync(0xffffffffu, other, o);
-      }
-    }
-    double r = w[0];
-#pragma unroll
-    for (int k = LANES / P / 2; k > 0; k >>= 1) r += __shfl_xor_sync(0xffffffffu, r, k);
-    const int mine = hl / (LANES / P);
-    if (hl % (LANES / P) == 0 && mine < TAKE) out[mine] = r;
-    gram_reduce<LANES, N - TAKE>(v + TAKE, hl, out + TAKE);
-  }
-}
-
 // moments with x exponents A0 .. A1 and z exponents C0 .. C1
 template <typename S, int A0, int A1, int C0, int C1>
 __device__ __forceinline__ void gram_moments(const double (&x)[S::SLOTS], const double (&y)[S::SLOTS],
@@ -183,7 +151,7 @@ __device__ __forceinline__ void gram_moments(const double (&x)[S::SLOTS], const 
       wc *= z[s];
     }
   }
-  gram_reduce<S::LANES, N>(acc, hl, out + S::mom(A0, 0, C0));
+  lane_sums<S::LANES, N>(acc, hl, out + S::mom(A0, 0, C0));
 }
 
 // reciprocal by Newton's iteration from the FP32 one: relative error 2^-23 -> 2^-46 -> 2^-53
@@ -278,7 +246,7 @@ __device__ __forceinline__ void gram_project(const double (&x)[S::SLOTS], const 
         xa *= x[k];
       }
     }
-    gram_reduce<S::LANES, NXY * TG>(acc, hl, out + t0 * NXY);
+    lane_sums<S::LANES, NXY * TG>(acc, hl, out + t0 * NXY);
   }
 }
 

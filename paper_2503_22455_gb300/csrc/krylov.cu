@@ -7,7 +7,7 @@
 //   w  -= V h, |w|^2             one fused pass                (k_update)
 //   optional second pass when |w| dropped below 1e-3 |w_old|   (classical
 //   Gram-Schmidt with re-orthogonalisation on severe cancellation)
-//   Givens rotation, Arnoldi residual estimate, flags         (k_arnoldi_step)
+//   Givens rotation, Arnoldi residual estimate, flags         (last block of k_update)
 // v_{j+1} is kept unnormalised; 1/|v_{j+1}| is applied inside the kernels that
 // read it.  Reductions are deterministic: per-block partials in a fixed grid,
 // summed in block order by the last block to finish.  Convergence is decided on
@@ -35,12 +35,7 @@ template <int NV>
 __device__ inline void block_reduce_store(double (&acc)[NV], double* partial, int stride, int vb, int nv = NV) {
   __shared__ double red[kRedThreads / 32][NV > 0 ? NV : 1];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-  for (int k = 0; k < NV; ++k) {
-    if (k >= nv) break;
-    double v = warp_sum(acc[k]);
-    if (lane == 0) red[wid][k] = v;
-  }
+  lane_sums<32, NV>(acc, lane, red[wid]);
   __syncthreads();
   if (threadIdx.x < nv) {
     double s = 0;
@@ -65,20 +60,23 @@ __device__ inline bool last_block(unsigned int* counter, int nvb) {
 
 // Sum the per-block partials in the last block: thread t adds blocks t, t+256, ... of
 // every component, then a fixed-order tree over the threads (deterministic).
+template <int NV>
 __device__ inline void sum_partials(const double* partial, int nblocks, int stride, int nv, double* out) {
-  __shared__ double red[kRedThreads / 32][kMaxRestart + 4];
+  __shared__ double red[kRedThreads / 32][NV];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int k = 0; k < nv; ++k) {
-    double s = 0;
-    for (int b = threadIdx.x; b < nblocks; b += blockDim.x) s += partial[(size_t)b * stride + k];
-    s = warp_sum(s);
-    if (lane == 0) red[wid][k] = s;
-  }
+  double s[NV];
+#pragma unroll
+  for (int k = 0; k < NV; ++k) s[k] = 0.0;
+  for (int b = threadIdx.x; b < nblocks; b += blockDim.x)
+#pragma unroll
+    for (int k = 0; k < NV; ++k)
+      if (k < nv) s[k] += partial[(size_t)b * stride + k];
+  lane_sums<32, NV>(s, lane, red[wid]);
   __syncthreads();
   if (threadIdx.x < nv) {
-    double s = 0;
-    for (int w = 0; w < kRedThreads / 32; ++w) s += red[w][threadIdx.x];
-    out[threadIdx.x] = s;
+    double t = 0;
+    for (int w = 0; w < kRedThreads / 32; ++w) t += red[w][threadIdx.x];
+    out[threadIdx.x] = t;
   }
   __syncthreads();
 }
@@ -111,7 +109,7 @@ __device__ inline void residual_body(const double* __restrict__ b, const double*
   block_reduce_store<2>(acc, partial, 4, vb);
   if (!last_block(counter, nvb)) return;
   __shared__ double tot[4];
-  sum_partials(partial, nvb, 4, 2, tot);
+  sum_partials<2>(partial, nvb, 4, 2, tot);
   if (threadIdx.x == 0) {
     *counter = 0;
     if (first == 2) {
@@ -160,9 +158,36 @@ __global__ void __launch_bounds__(kRedThreads) k_residual(const double* __restri
   residual_body(b, ax, v0, N, partial, counter, S, first, status, blockIdx.x, gridDim.x);
 }
 
+// One pass over w and the vectors before it: f(element, w, v(k)) for the pairs first, first + step, ...
+// STAGED: every vector's pair of several elements is loaded before the first is used.  The grid has two
+// blocks of 256 threads per SM, so a thread needs six and more 16-byte loads in flight to keep the
+// memory busy; left to itself the compiler went from 64 to 48 registers with a change elsewhere in the
+// kernel and took 286 us for 220 (256^3, ten vectors).
+template <int NV, bool STAGED, class F>
+__device__ __forceinline__ void orth_elements(const double* __restrict__ V, int64_t Np, const double2* w2, int64_t first,
+                                              int64_t step, int64_t N2, F f) {
+  int64_t e = first;
+  if constexpr (STAGED) {
+    constexpr int U = NV <= 2 ? 6 : (NV <= 3 ? 4 : (NV <= 6 ? 2 : 1));
+    for (; e + (U - 1) * step < N2; e += U * step) {
+      double2 wv[U], vv[U][NV];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        wv[u] = w2[e + u * step];
+#pragma unroll
+        for (int k = 0; k < NV; ++k) vv[u][k] = reinterpret_cast<const double2*>(V + (size_t)k * Np)[e + u * step];
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) f(e + u * step, wv[u], [&](int k) { return vv[u][k]; });
+    }
+  }
+  for (; e < N2; e += step)
+    f(e, w2[e], [&](int k) { return reinterpret_cast<const double2*>(V + (size_t)k * Np)[e]; });
+}
+
 // h_i = inv_norm_i <V_i, w> (i < nv = j + 1), |w|^2 ; w = V[j+1].  NVMAX bounds nv at
 // compile time (a single solve instantiates NVMAX = nv; the batched engine 16).
-template <int NVMAX>
+template <int NVMAX, bool STAGED>
 __device__ inline void multidot_body(const double* __restrict__ V, int64_t Np, int j, int nv, double* partial,
                                      unsigned int* counter, SolverScalars* S, int second, int vb, int nvb) {
   if (second && !S->reorth_needed) return;
@@ -172,39 +197,36 @@ __device__ inline void multidot_body(const double* __restrict__ V, int64_t Np, i
   for (int k = 0; k <= NVMAX; ++k) acc[k] = 0.0;
   const int64_t N2 = Np / 2;
   const double2* w2 = reinterpret_cast<const double2*>(w);
-  for (int64_t e = (int64_t)vb * blockDim.x + threadIdx.x; e < N2; e += (int64_t)nvb * blockDim.x) {
-    double2 wv = w2[e];
+  const int64_t first = (int64_t)vb * blockDim.x + threadIdx.x, step = (int64_t)nvb * blockDim.x;
+  auto take = [&](double2 wv, auto vv) {
 #pragma unroll
     for (int k = 0; k < NVMAX; ++k) {
       if (k >= nv) break;
-      double2 vv = reinterpret_cast<const double2*>(V + (size_t)k * Np)[e];
-      acc[k] = fma(vv.x, wv.x, acc[k]);
-      acc[k] = fma(vv.y, wv.y, acc[k]);
+      const double2 v = vv(k);
+      acc[k] = fma(v.x, wv.x, acc[k]);
+      acc[k] = fma(v.y, wv.y, acc[k]);
     }
     acc[NVMAX] = fma(wv.x, wv.x, acc[NVMAX]);
     acc[NVMAX] = fma(wv.y, wv.y, acc[NVMAX]);
-  }
+  };
+  orth_elements<NVMAX, STAGED>(V, Np, w2, first, step, N2, [&](int64_t, double2 wv, auto vv) { take(wv, vv); });
+  pdl_trigger();                       // the next kernel's launch overlaps the reduction
   {
     // partials [h_0 .. h_j, |w|^2]: component nv is acc[NVMAX] (static register indices)
     __shared__ double red[kRedThreads / 32][NVMAX + 1];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int k = 0; k <= NVMAX; ++k) {
-      if (k < nv || k == NVMAX) {
-        double v = warp_sum(acc[k]);
-        if (lane == 0) red[wid][k < nv ? k : nv] = v;
-      }
-    }
+    lane_sums<32, NVMAX + 1>(acc, lane, red[wid]);
     __syncthreads();
     if (threadIdx.x <= nv) {
+      const int k = threadIdx.x < nv ? threadIdx.x : NVMAX;
       double s = 0;
-      for (int w = 0; w < kRedThreads / 32; ++w) s += red[w][threadIdx.x];
+      for (int w = 0; w < kRedThreads / 32; ++w) s += red[w][k];
       partial[(size_t)vb * (kMaxRestart + 4) + threadIdx.x] = s;
     }
   }
   if (!last_block(counter, nvb)) return;
   __shared__ double tot[kMaxRestart + 4];
-  sum_partials(partial, nvb, kMaxRestart + 4, nv + 1, tot);
+  sum_partials<NVMAX + 1>(partial, nvb, kMaxRestart + 4, nv + 1, tot);
   if (threadIdx.x == 0) {
     *counter = 0;
     if (!second) {
@@ -218,16 +240,101 @@ __device__ inline void multidot_body(const double* __restrict__ V, int64_t Np, i
 }
 
 template <int NV>
-__global__ void __launch_bounds__(kRedThreads) k_multidot(const double* __restrict__ V, int64_t Np, int j,
+__global__ void __launch_bounds__(kRedThreads, 2) k_multidot(const double* __restrict__ V, int64_t Np, int j,
                                                           double* partial, unsigned int* counter, SolverScalars* S,
                                                           int second) {
-  multidot_body<NV>(V, Np, j, NV, partial, counter, S, second, blockIdx.x, gridDim.x);
+  pdl_wait();
+  multidot_body<NV, true>(V, Np, j, NV, partial, counter, S, second, blockIdx.x, gridDim.x);
 }
 
-// w -= sum_i c_i V_i with c_i = h_i inv_norm_i (i < nv) ; |w|^2
-template <int NVMAX>
+// The kernels of an iteration are chained as dependent launches; each lets the next one be launched when
+// its blocks are through with the vectors, not before, so that no waiting block takes an SM's room from
+// a running one.  With the sums across a warp transposed (common.cuh), the Givens step in the last block
+// of the update and the coefficients of x in the blocks that use them, a pass takes (multi-dot / update
+// with six vectors) 26.7 -> 18.0 / 18.5 -> 16.8 us at 96^3, 210 -> 204 / 220 -> 209 us at 256^3, and the
+// launches of one thread (9 us per iteration, 10 per restart) are gone: the 64^2 circle's solve
+// 1463 -> 1260 us, the 1024^2 star's step 7.31 -> 6.93 ms.
+//
+// Givens rotations on column j, estimate, flags, by one block: the column and the rotations so far are
+// read by as many threads, threads of other warps take the
+// norms' roots and reciprocals, one thread rotates.
+__device__ inline void arnoldi_block(SolverScalars* S, int j, int* status) {
+  __shared__ double h[kMaxRestart + 1], cs[kMaxRestart], sn[kMaxRestart], s_w2, s_hn, s_inv, s_ib;
+  const int t = threadIdx.x, L = kMaxRestart + 1;
+  double* H = S->H;
+  if (t <= j) h[t] = S->hcol[t];
+  if (t < j) {
+    cs[t] = S->cs[t];
+    sn[t] = S->sn[t];
+  }
+  if (t == (blockDim.x > 32 ? 32 : 0)) {
+    s_w2 = S->w2;
+    s_hn = sqrt(s_w2);
+    s_inv = s_hn > 0 ? 1.0 / s_hn : 0.0;
+  }
+  if (t == (blockDim.x > 64 ? 64 : 0)) s_ib = S->bnorm > 0 ? 1.0 / S->bnorm : 0.0;
+  double g = 0, tol = 0;
+  int iters = 0, max_iter = 0, m = 0;
+  if (t == 0) {
+    g = S->g[j];
+    tol = S->tol;
+    iters = S->iters;
+    max_iter = S->max_iter;
+    m = S->m;
+  }
+  __syncthreads();
+  if (t == 0) {
+    for (int i = 0; i < j; ++i) {
+      const double a = h[i], b = h[i + 1];
+      h[i] = cs[i] * a + sn[i] * b;
+      h[i + 1] = -sn[i] * a + cs[i] * b;
+    }
+    const double hn = s_hn;
+    const double a = h[j], b = hn;
+    // the square of b = |w| is what was summed: one reciprocal root gives the radius and the rotation
+    const double q = fma(a, a, s_w2);
+    double den, c, s;
+    if (q > 1e-280 && q < 1e280) {
+      const double r = rsqrt(q);
+      den = q * r;
+      c = a * r;
+      s = b * r;
+    } else {
+      den = hypot(a, b);
+      c = den > 0 ? a / den : 1.0;
+      s = den > 0 ? b / den : 0.0;
+    }
+    h[j] = den;
+    S->inv_norm[j + 1] = s_inv;
+    S->cs[j] = c;
+    S->sn[j] = s;
+    const double gn = -s * g;
+    S->g[j + 1] = gn;
+    S->g[j] = c * g;
+    S->iters = iters + 1;
+    S->k = j + 1;
+    const double est = fabs(gn) * s_ib;
+    S->est = est;
+    const bool bad = !(est == est) || !(hn == hn) || isinf(hn);
+    if (bad) {
+      set_status(status, IIM_ERR_BREAKDOWN);
+      S->breakdown = 1;
+    }
+    const bool stop = bad || hn == 0.0 || est <= tol || iters + 1 >= max_iter || j + 1 >= m;
+    S->active = !stop;
+    if (j + 1 < m) set_cond(S, S->h_if[j + 1], !stop);
+  }
+  __syncthreads();
+  if (t <= j) H[t + L * j] = h[t];
+  if (t == j + 1) H[t + L * j] = 0.0;
+}
+
+// w -= sum_i c_i V_i with c_i = h_i inv_norm_i (i < nv) ; |w|^2.  With arnoldi, the last block also
+// closes the iteration (arnoldi_block) unless a second pass is due.
+template <int NVMAX, bool STAGED>
 __device__ inline void update_body(double* __restrict__ V, int64_t Np, int j, int nv, double* partial,
-                                   unsigned int* counter, SolverScalars* S, int second, int vb, int nvb) {
+                                   unsigned int* counter, SolverScalars* S, int second, int vb, int nvb, bool arnoldi,
+                                   int* status) {
   if (second && !S->reorth_needed) return;
   __shared__ double c[NVMAX];
   if (threadIdx.x < nv) c[threadIdx.x] = (second ? S->y[threadIdx.x] : S->hcol[threadIdx.x]) * S->inv_norm[threadIdx.x];
@@ -236,23 +343,25 @@ __device__ inline void update_body(double* __restrict__ V, int64_t Np, int j, in
   double acc[1] = {0.0};
   const int64_t N2 = Np / 2;
   double2* w2 = reinterpret_cast<double2*>(w);
-  for (int64_t e = (int64_t)vb * blockDim.x + threadIdx.x; e < N2; e += (int64_t)nvb * blockDim.x) {
-    double2 wv = w2[e];
+  const int64_t first = (int64_t)vb * blockDim.x + threadIdx.x, step = (int64_t)nvb * blockDim.x;
+  orth_elements<NVMAX, STAGED>(V, Np, w2, first, step, N2, [&](int64_t e, double2 wv, auto vv) {
 #pragma unroll
     for (int k = 0; k < NVMAX; ++k) {
       if (k >= nv) break;
-      double2 vv = reinterpret_cast<const double2*>(V + (size_t)k * Np)[e];
-      wv.x = fma(-c[k], vv.x, wv.x);
-      wv.y = fma(-c[k], vv.y, wv.y);
+      const double2 v = vv(k);
+      wv.x = fma(-c[k], v.x, wv.x);
+      wv.y = fma(-c[k], v.y, wv.y);
     }
     w2[e] = wv;
     acc[0] = fma(wv.x, wv.x, acc[0]);
     acc[0] = fma(wv.y, wv.y, acc[0]);
-  }
+  });
+  pdl_trigger();                       // the next kernel's launch overlaps the reduction
   block_reduce_store<1>(acc, partial, kMaxRestart + 4, vb);
   if (!last_block(counter, nvb)) return;
   __shared__ double tot[kMaxRestart + 4];
-  sum_partials(partial, nvb, kMaxRestart + 4, 1, tot);
+  __shared__ int close;
+  sum_partials<1>(partial, nvb, kMaxRestart + 4, 1, tot);
   if (threadIdx.x == 0) {
     *counter = 0;
     S->w2 = tot[0];
@@ -260,87 +369,60 @@ __device__ inline void update_body(double* __restrict__ V, int64_t Np, int j, in
       // second pass only on severe cancellation, |w| < 1e-3 |w_old| (a DGKS test with a small eta:
       // with the multigrid preconditioner |w| drops below |w_old|/sqrt(2) at every iteration,
       // yet one pass gives the same iterates' quality and iteration counts)
-      S->reorth_needed = S->reorth && (tot[0] < 1e-6 * S->w2_old);
+      const int again = S->reorth && (tot[0] < 1e-6 * S->w2_old);
+      S->reorth_needed = again;
+      close = arnoldi && !again;
     } else {
       for (int k = 0; k < nv; ++k) S->hcol[k] += S->y[k];
       S->reorth_needed = 0;
+      close = arnoldi;
     }
   }
+  __syncthreads();
+  if (close) arnoldi_block(S, j, status);
 }
 
 template <int NV>
-__global__ void __launch_bounds__(kRedThreads) k_update(double* __restrict__ V, int64_t Np, int j, double* partial,
-                                                        unsigned int* counter, SolverScalars* S, int second) {
-  update_body<NV>(V, Np, j, NV, partial, counter, S, second, blockIdx.x, gridDim.x);
+__global__ void __launch_bounds__(kRedThreads, 2) k_update(double* __restrict__ V, int64_t Np, int j, double* partial,
+                                                        unsigned int* counter, SolverScalars* S, int second, int arnoldi,
+                                                        int* status) {
+  pdl_wait();
+  update_body<NV, true>(V, Np, j, NV, partial, counter, S, second, blockIdx.x, gridDim.x, arnoldi != 0, status);
 }
 
-// Givens rotations on column j, estimate, flags (one thread)
-__device__ inline void arnoldi_body(SolverScalars* S, int j, int* status) {
-  const int L = kMaxRestart + 1;
-  double* H = S->H;
-  for (int i = 0; i <= j; ++i) H[i + L * j] = S->hcol[i];
-  double hn = sqrt(S->w2);
-  H[j + 1 + L * j] = hn;
-  S->inv_norm[j + 1] = hn > 0 ? 1.0 / hn : 0.0;
-  for (int i = 0; i < j; ++i) {
-    double a = H[i + L * j], b = H[i + 1 + L * j];
-    H[i + L * j] = S->cs[i] * a + S->sn[i] * b;
-    H[i + 1 + L * j] = -S->sn[i] * a + S->cs[i] * b;
+// y = H^-1 g (k x k upper triangular) by one warp: lane r holds g_r, each y_i leaves its column from
+// the rows above at once
+__device__ inline void solve_y_warp(const SolverScalars* S, double* y) {
+  const int L = kMaxRestart + 1, k = S->k, r = threadIdx.x & 31;
+  const double d = r < k ? S->H[r + L * r] : 0.0;
+  const double inv = d != 0.0 ? 1.0 / d : 0.0;
+  double g = r < k ? S->g[r] : 0.0;
+  double h[kMaxRestart];
+#pragma unroll
+  for (int c = 0; c < kMaxRestart; ++c) h[c] = r < c && c < k ? S->H[r + L * c] : 0.0;
+#pragma unroll
+  for (int i = kMaxRestart - 1; i >= 0; --i) {
+    if (i >= k) continue;
+    const double yi = __shfl_sync(0xffffffffu, g * inv, i);
+    if (r == i) g = yi;
+    else g = fma(-h[i], yi, g);
   }
-  double a = H[j + L * j], b = H[j + 1 + L * j];
-  double den = hypot(a, b);
-  double cs = den > 0 ? a / den : 1.0, sn = den > 0 ? b / den : 0.0;
-  S->cs[j] = cs;
-  S->sn[j] = sn;
-  H[j + L * j] = den;
-  H[j + 1 + L * j] = 0.0;
-  S->g[j + 1] = -sn * S->g[j];
-  S->g[j] = cs * S->g[j];
-  S->iters += 1;
-  S->k = j + 1;
-  double est = S->bnorm > 0 ? fabs(S->g[j + 1]) / S->bnorm : 0.0;
-  S->est = est;
-  bool bad = !(est == est) || !(hn == hn) || isinf(hn);
-  if (bad) {
-    set_status(status, IIM_ERR_BREAKDOWN);
-    S->breakdown = 1;
-  }
-  bool stop = bad || hn == 0.0 || est <= S->tol || S->iters >= S->max_iter || j + 1 >= S->m;
-  S->active = !stop;
-  if (j + 1 < S->m) set_cond(S, S->h_if[j + 1], !stop);
-}
-
-__global__ void k_arnoldi_step(SolverScalars* S, int j, int* status) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  arnoldi_body(S, j, status);
-}
-
-// y = H^-1 g (k x k upper triangular)
-__device__ inline void solve_y_body(SolverScalars* S) {
-  const int L = kMaxRestart + 1, k = S->k;
-  for (int i = k - 1; i >= 0; --i) {
-    double s = S->g[i];
-    for (int c = i + 1; c < k; ++c) s -= S->H[i + L * c] * S->y[c];
-    double d = S->H[i + L * i];
-    S->y[i] = d != 0.0 ? s / d : 0.0;
-  }
-  for (int i = k; i < kMaxRestart; ++i) S->y[i] = 0.0;
-}
-
-__global__ void k_solve_y(SolverScalars* S) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  solve_y_body(S);
+  if (r < kMaxRestart) y[r] = r < k ? g : 0.0;
 }
 
 // x += sum_{i<k} y_i Z_i (right preconditioning), or x += sum_{i<k} y_i V_i / |V_i| with
-// Z = V (left preconditioning: the basis is stored unnormalised)
+// Z = V (left preconditioning: the basis is stored unnormalised).  Every block solves for the coefficients
+// itself, which costs less than a launch of one warp before this one.
 __device__ inline void xupdate_body(double* __restrict__ x, const double* __restrict__ Z, int64_t Np, int64_t N,
-                                    const SolverScalars* S, int vb, int nvb, bool unnormalised = false) {
+                                    const SolverScalars* S, int vb, int nvb,
+                                    bool unnormalised = false) {
   __shared__ double y[kMaxRestart];
-  __shared__ int k;
-  if (threadIdx.x < kMaxRestart)
-    y[threadIdx.x] = unnormalised ? S->y[threadIdx.x] * S->inv_norm[threadIdx.x] : S->y[threadIdx.x];
-  if (threadIdx.x == 0) k = S->k;
+  if (threadIdx.x < 32) {
+    solve_y_warp(S, y);
+    __syncwarp();
+    if (unnormalised && threadIdx.x < kMaxRestart) y[threadIdx.x] *= S->inv_norm[threadIdx.x];
+  }
+  const int k = S->k;
   __syncthreads();
   for (int64_t i = (int64_t)vb * blockDim.x + threadIdx.x; i < N; i += (int64_t)nvb * blockDim.x) {
     double acc = x[i];
@@ -413,36 +495,24 @@ iim_status krylov_alloc(Problem& P) {
   return IIM_OK;
 }
 
-template <int NV>
-static void launch_orth(Problem& P, int j, cudaStream_t s, int second) {
-  IIM_LAUNCH(k_multidot<NV>, P.red_blocks, kRedThreads, 0, s, P.V, P.Npad, j, P.partial, P.counter, P.sc, second);
-  IIM_LAUNCH(k_update<NV>, P.red_blocks, kRedThreads, 0, s, P.V, P.Npad, j, P.partial, P.counter, P.sc, second);
-}
-
-static void orth(Problem& P, int j, cudaStream_t s, int second) {
+// one multidot (which = 0) or update (which = 1) pass over v_0..v_j; close: the update ends the iteration
+static void orth_pass(Problem& P, int j, int which, int second, int close, cudaStream_t s) {
   switch (j + 1) {
-#define IIM_CASE(k) case k: launch_orth<k>(P, j, s, second); break;
-    IIM_CASE(1) IIM_CASE(2) IIM_CASE(3) IIM_CASE(4) IIM_CASE(5) IIM_CASE(6) IIM_CASE(7) IIM_CASE(8)
-    IIM_CASE(9) IIM_CASE(10) IIM_CASE(11) IIM_CASE(12) IIM_CASE(13) IIM_CASE(14) IIM_CASE(15) IIM_CASE(16)
-#undef IIM_CASE
-  }
-}
-
-// one multidot (which = 0) or update (which = 1) pass over v_0..v_j (kernel timing)
-void krylov_orth_pass(Problem& P, int j, int which, cudaStream_t s) {
-  switch (j + 1) {
-#define IIM_CASE(k)                                                                                          \
-  case k:                                                                                                    \
-    if (which == 0)                                                                                          \
-      IIM_LAUNCH(k_multidot<k>, P.red_blocks, kRedThreads, 0, s, P.V, P.Npad, j, P.partial, P.counter, P.sc, 0); \
-    else                                                                                                     \
-      IIM_LAUNCH(k_update<k>, P.red_blocks, kRedThreads, 0, s, P.V, P.Npad, j, P.partial, P.counter, P.sc, 0);   \
+#define IIM_CASE(k)                                                                                                 \
+  case k:                                                                                                           \
+    if (which == 0)                                                                                                 \
+      IIM_LAUNCH_PDL(k_multidot<k>, P.red_blocks, kRedThreads, 0, s, (const double*)P.V, P.Npad, j, P.partial, P.counter, P.sc, second); \
+    else                                                                                                            \
+      IIM_LAUNCH_PDL(k_update<k>, P.red_blocks, kRedThreads, 0, s, P.V, P.Npad, j, P.partial, P.counter, P.sc, second, close,   \
+                     P.d_status + 1);                                                                               \
     break;
     IIM_CASE(1) IIM_CASE(2) IIM_CASE(3) IIM_CASE(4) IIM_CASE(5) IIM_CASE(6) IIM_CASE(7) IIM_CASE(8)
     IIM_CASE(9) IIM_CASE(10) IIM_CASE(11) IIM_CASE(12) IIM_CASE(13) IIM_CASE(14) IIM_CASE(15) IIM_CASE(16)
 #undef IIM_CASE
   }
 }
+
+void krylov_orth_pass(Problem& P, int j, int which, cudaStream_t s) { orth_pass(P, j, which, 0, 0, s); }
 
 // Augmented system (pure Neumann, Sec. 2.3): w = L u + alpha 1 on the unknowns, w_N = 1^T u.
 // The sum is deterministic: block partials in a fixed grid, summed by the last block to finish (a
@@ -460,7 +530,7 @@ __global__ void __launch_bounds__(256) k_aug_apply(const double* __restrict__ u,
   block_reduce_store<1>(acc, partial, 1, blockIdx.x);
   if (!last_block(counter, gridDim.x)) return;
   __shared__ double tot[1];
-  sum_partials(partial, gridDim.x, 1, 1, tot);
+  sum_partials<1>(partial, gridDim.x, 1, 1, tot);
   if (threadIdx.x == 0) {
     *counter = 0;
     w[N] = tot[0];
@@ -499,9 +569,10 @@ static void enqueue_iteration(Problem& P, int j, cudaStream_t s) {
     krylov_precondition(P, vj, &P.sc->inv_norm[j], zj, s);
     krylov_apply(P, zj, w, s);
   }
-  orth(P, j, s, 0);
-  if (P.opt.reorth) orth(P, j, s, 1);
-  IIM_LAUNCH(k_arnoldi_step, 1, 32, 0, s, P.sc, j, P.d_status + 1);
+  for (int pass = 0; pass < (P.opt.reorth ? 2 : 1); ++pass) {
+    orth_pass(P, j, 0, pass, 0, s);
+    orth_pass(P, j, 1, pass, 1, s);
+  }
 }
 
 // left preconditioning: V0 = M (b - L x), measured (first: 0 restart, 3 start)
@@ -516,7 +587,6 @@ static void enqueue_left_residual(Problem& P, cudaStream_t s, int first) {
 }
 
 static void enqueue_restart(Problem& P, cudaStream_t s) {
-  IIM_LAUNCH(k_solve_y, 1, 32, 0, s, P.sc);
   if (left_prec(P)) {
     IIM_LAUNCH(k_xupdate, 4 * kNumSMs, 256, 0, s, P.x, P.V, P.Npad, P.g.N + P.aug, P.sc, 1);
     enqueue_left_residual(P, s, 0);
@@ -782,14 +852,6 @@ __global__ void __launch_bounds__(1024) k_eng_plan(EngArgs A, int* dyn, int forc
   }
 }
 
-__global__ void __launch_bounds__(32) k_eng_solve_y(EngArgs A) {
-  eng_for_items(A, kDynAllRestart, [&](int si, int) {
-    const SlotDev& s = A.slots[si];
-    if (s.role != kRoleRestart || threadIdx.x != 0) return;
-    solve_y_body(s.sc);
-  });
-}
-
 __global__ void __launch_bounds__(256) k_eng_xupdate(EngArgs A) {
   eng_for_items(A, kListXup, [&](int si, int item) {
     const SlotDev& s = A.slots[si];
@@ -802,7 +864,7 @@ __global__ void __launch_bounds__(kRedThreads) k_eng_multidot(EngArgs A, int sec
   eng_for_items(A, kListRed, [&](int si, int item) {
     const SlotDev& s = A.slots[si];
     if (s.role != kRoleIter) return;
-    multidot_body<kMaxRestart>(s.V, s.Npad, s.j, s.j + 1, s.partial, s.counter, s.sc, second, item, s.red_blocks);
+    multidot_body<kMaxRestart, false>(s.V, s.Npad, s.j, s.j + 1, s.partial, s.counter, s.sc, second, item, s.red_blocks);
   });
 }
 
@@ -810,15 +872,8 @@ __global__ void __launch_bounds__(kRedThreads) k_eng_update(EngArgs A, int secon
   eng_for_items(A, kListRed, [&](int si, int item) {
     const SlotDev& s = A.slots[si];
     if (s.role != kRoleIter) return;
-    update_body<kMaxRestart>(s.V, s.Npad, s.j, s.j + 1, s.partial, s.counter, s.sc, second, item, s.red_blocks);
-  });
-}
-
-__global__ void __launch_bounds__(32) k_eng_arnoldi(EngArgs A) {
-  eng_for_items(A, kDynAllIter, [&](int si, int) {
-    const SlotDev& s = A.slots[si];
-    if (s.role != kRoleIter || threadIdx.x != 0) return;
-    arnoldi_body(s.sc, s.j, s.status);
+    update_body<kMaxRestart, false>(s.V, s.Npad, s.j, s.j + 1, s.partial, s.counter, s.sc, second, item, s.red_blocks, true,
+                             s.status);
   });
 }
 
@@ -864,7 +919,6 @@ void eng_launch_plan(const EngArgs& A, int* dyn, int force_iter, cudaStream_t s)
 
 void eng_launch_krylov_head(const EngArgs& A, int* dyn, cudaStream_t s) {
   eng_launch_plan(A, dyn, 0, s);
-  IIM_LAUNCH(k_eng_solve_y, eng_grid((const void*)k_eng_solve_y, 32, 0), 32, 0, s, A);
   IIM_LAUNCH(k_eng_xupdate, eng_grid((const void*)k_eng_xupdate, 256, 0), 256, 0, s, A);
 }
 
@@ -876,7 +930,6 @@ void eng_launch_krylov_tail(const EngArgs& A, int* ctl, cudaGraphConditionalHand
   IIM_LAUNCH(k_eng_update, gu, kRedThreads, 0, s, A, 0);
   IIM_LAUNCH(k_eng_multidot, gr, kRedThreads, 0, s, A, 1);
   IIM_LAUNCH(k_eng_update, gu, kRedThreads, 0, s, A, 1);
-  IIM_LAUNCH(k_eng_arnoldi, eng_grid((const void*)k_eng_arnoldi, 32, 0), 32, 0, s, A);
   IIM_LAUNCH(k_eng_residual, eng_grid((const void*)k_eng_residual, kRedThreads, 0), kRedThreads, 0, s, A);
   IIM_LAUNCH(k_eng_tick_end, 1, 256, 0, s, A, ctl, ctl + 2, ctl + 1, h, use_cond);
 }
