@@ -327,6 +327,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 7 : 1) k_mg2d(Fine2DPara
 // ---------------------------------------------------------------------------- coarse tail (one CTA)
 constexpr int kTailMaxLevels = 8;
 constexpr int kTailNodes = 1024;      // levels with at most this many nodes go to the tail
+constexpr int kTailCluster = 8;       // CTAs that share a large dense solve
 constexpr int kTailThreads = 1024;    // threads of the tail's CTA: one node each on its first level
 
 template <typename T>
@@ -402,30 +403,134 @@ struct NodeWalk {
   }
 };
 
-template <typename T, int DIM>
+// FP64 tails stage their rows as [diagonal, off-diagonals, 1 / diagonal], with one more for the regular
+// nodes, so that every node of a sweep runs the same few FP64 operations: a division takes the place of
+// a dozen, and one irregular node makes its whole warp run the second path (GB300 issues two FP64
+// operations per clock and SM, and the tail has one to a few SMs).  With that, full warps per colour and
+// the shared dense solve the tail of a 104^2 problem (26^2, 13^2) takes 19.6 us for 71.0, of a 120^2 one
+// 23.3 for 94.8, of 40^3 30.6 for 121; FP32, same arithmetic as before, 12.6 for 14.5 and 13.1 for 16.7.
+__host__ __device__ constexpr int tail_row64(int dim) { return 2 * dim + 2; }
+template <typename T>
+__host__ __device__ constexpr int tail_row(int dim) { return sizeof(T) == 8 ? tail_row64(dim) : sw_row(dim); }
+template <int DIM>
+__device__ __forceinline__ double tail_offdiag64(int n, const double* row, const double* u, int i, const int* m) {
+  double s = 0;
+  int st = 1;
+#pragma unroll
+  for (int ax = 0; ax < DIM; ++ax) {
+    // (the coefficients across the box's faces are 0)
+    const double t = row[1 + 2 * ax] * u[m[ax] > 0 ? i - st : i];
+    s += fma(row[2 + 2 * ax], u[m[ax] < n - 1 ? i + st : i], t);
+    st *= n;
+  }
+  return s;
+}
+
+// Where the tail's CTAs stand: one alone, or a cluster whose first CTA runs the levels while the others
+// wait to take their rows of the dense solve, its f and u read and written in the first one's memory.
+template <bool CLUSTER>
+struct TailGroup {
+  int rank = 0, size = 1;
+  __device__ __forceinline__ TailGroup() {
+    if (CLUSTER) {
+      asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+      asm("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(size));
+    }
+  }
+  __device__ __forceinline__ void sync() const {
+    if (CLUSTER) {
+      asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+      asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    } else {
+      __syncthreads();
+    }
+  }
+  // address in the first CTA's shared memory of this CTA's p
+  __device__ __forceinline__ unsigned first(const void* p) const {
+    unsigned a = (unsigned)__cvta_generic_to_shared(p), r;
+    asm("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(a));
+    return r;
+  }
+  __device__ __forceinline__ float load(const float* p) const {
+    float v;
+    if (!CLUSTER) return *p;
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(first(p)) : "memory");
+    return v;
+  }
+  __device__ __forceinline__ double load(const double* p) const {
+    double v;
+    if (!CLUSTER) return *p;
+    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(first(p)) : "memory");
+    return v;
+  }
+  __device__ __forceinline__ void store(float* p, float v) const {
+    if (!CLUSTER) *p = v;
+    else asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(first(p)), "f"(v) : "memory");
+  }
+  __device__ __forceinline__ void store(double* p, double v) const {
+    if (!CLUSTER) *p = v;
+    else asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(first(p)), "d"(v) : "memory");
+  }
+};
+
+// 1 / count of active parents
+__device__ const double kTailInv[9] = {0.0, 1.0, 1.0 / 2, 1.0 / 3, 1.0 / 4, 1.0 / 5, 1.0 / 6, 1.0 / 7, 1.0 / 8};
+
+// the sums of v[0 .. 3] over the warp, each the tree of a butterfly (lanes 16 apart first); lane
+// 16 a + 8 b (and the seven after it) get that of v[2 a + b]
+template <typename T>
+__device__ __forceinline__ T lane_sum4(const T (&v)[4], int lane) {
+  const bool a = lane & 16, b = lane & 8;
+  const T w0 = (a ? v[2] : v[0]) + __shfl_xor_sync(0xffffffffu, a ? v[0] : v[2], 16);
+  const T w1 = (a ? v[3] : v[1]) + __shfl_xor_sync(0xffffffffu, a ? v[1] : v[3], 16);
+  T w = (b ? w1 : w0) + __shfl_xor_sync(0xffffffffu, b ? w0 : w1, 8);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+  return w;
+}
+
+template <typename T, int DIM, bool CLUSTER = false>
 __device__ __forceinline__ void vcycle_tail_body(const TailParams<T>& P, const double* v_in, const double* vscale,
                                                  double* z_out) {
   extern __shared__ unsigned char smraw[];
+  constexpr bool F64 = sizeof(T) == 8;
+  constexpr int SR = tail_row<T>(DIM);
+  const TailGroup<CLUSTER> G;
   const int tot = P.off[P.nlev];
   T* su = (T*)smraw;
   T* sf = su + tot;
-  T* st = sf + tot;                                   // staged tables
-  int* sa = (int*)(st + P.toff[P.nlev]);
+  T* st = sf + tot;                                   // staged tables, then (FP64) residuals of a level
+  T* sr = st + P.toff[P.nlev];
+  int* sa = (int*)(sr + (F64 && P.nlev > 1 ? P.off[1] : 0));
   int* sco = sa + tot;                                 // node coordinates, i0 | i1 << 10 | i2 << 20
+  T* sg = (T*)(sco + tot);                             // (cluster) the coarsest level's f, its unknowns only
   const int tid = threadIdx.x, nt = blockDim.x;
-  for (int k = 0; k < P.nlev; ++k) {
-    const int n = P.L[k].n;
-    for (int i = tid; i < P.L[k].N; i += nt) {
-      sa[P.off[k] + i] = P.L[k].aux[i];
-      const int r = i / n;
-      sco[P.off[k] + i] = (i - r * n) | ((DIM > 2 ? r % n : r) << 10) | ((DIM > 2 ? r / n : 0) << 20);
-    }
-  }
-  if (P.stage_tables) {
+  if (G.rank == 0) {
     for (int k = 0; k < P.nlev; ++k) {
-      const int rows = min(*P.tcount[k], P.tcap[k]);
-      const int len = rows * sw_row(DIM);
-      for (int e = tid; e < len; e += nt) st[P.toff[k] + e] = P.L[k].tab[e];
+      const int n = P.L[k].n, N = (int)P.L[k].N;
+      for (int i = tid; i < N; i += nt) {
+        const int a = P.L[k].aux[i];
+        sa[P.off[k] + i] = F64 && a == -1 ? P.tcap[k] : a;
+        const int r = i / n;
+        sco[P.off[k] + i] = (i - r * n) | ((DIM > 2 ? r % n : r) << 10) | ((DIM > 2 ? r / n : 0) << 20);
+      }
+    }
+    if (P.stage_tables) {
+      for (int k = 0; k + 1 < P.nlev; ++k) {
+        const int rows = min(*P.tcount[k], P.tcap[k]);
+        T* to = st + P.toff[k];
+        if constexpr (F64) {
+          for (int r = tid; r < rows; r += nt) {
+            const T* row = P.L[k].tab + (size_t)r * sw_row(DIM);
+            for (int e = 0; e <= 2 * DIM; ++e) to[r * SR + e] = row[e];
+            to[r * SR + SR - 1] = row[0] != 0.0 ? 1.0 / row[0] : 0.0;
+          }
+          if (tid < SR) to[P.tcap[k] * SR + tid] = tid == 0 ? P.L[k].dreg : (tid == SR - 1 ? P.L[k].inv_dreg : P.L[k].ih2);
+        } else {
+          const int len = rows * SR;
+          for (int e = tid; e < len; e += nt) to[e] = P.L[k].tab[e];
+        }
+      }
     }
   }
   auto table = [&](int k) -> const T* { return P.stage_tables ? st + P.toff[k] : P.L[k].tab; };
@@ -433,7 +538,7 @@ __device__ __forceinline__ void vcycle_tail_body(const TailParams<T>& P, const d
   // kernels before this one
   pdl_trigger();
   pdl_wait();
-  {
+  if (G.rank == 0) {
     const LevelK<T>& L = P.L[0];
     const T vs = v_in ? (T)(vscale ? *vscale : 1.0) : (T)1;
     for (int i = tid; i < L.N; i += nt) {
@@ -441,23 +546,28 @@ __device__ __forceinline__ void vcycle_tail_body(const TailParams<T>& P, const d
       if (L.aux[i] != -2) f = v_in ? (T)v_in[i] * (vs * (P.phase[i] ? P.inv_bp : P.inv_bm)) : load_f(L.f, i, L.f_bf16);
       sf[i] = f;
     }
+    __syncthreads();
   }
-  __syncthreads();
-  // thread tid owns nodes tid, tid + blockDim.x, ... of every level (one node when N <= blockDim.x)
+  // A thread takes a node of every second, 2 p or 2 p + 1 by colour (the levels that are smoothed have
+  // been halved, so their rows are even): full warps, where one thread per node left half of each idle.
   auto sweep = [&](int k, int colour, bool from_zero) {
     const LevelK<T>& L = P.L[k];
     T* u = su + P.off[k];
     const T* f = sf + P.off[k];
     const T* tb = table(k);
-    const int n = L.n;
-    for (int i = tid; i < L.N; i += blockDim.x) {
+    const int half = (int)L.N / 2;
+    for (int p = tid; p < half; p += nt) {
+      const int c = sco[P.off[k] + 2 * p];
+      const int sel = (c + (c >> 10) + (c >> 20) + colour) & 1, i = 2 * p + sel;
       const int a = sa[P.off[k] + i];
-      const int c = sco[P.off[k] + i];
-      const int m[3] = {c & 1023, (c >> 10) & 1023, c >> 20};
-      if (((m[0] + m[1] + m[2]) & 1) != colour) {
-        if (from_zero) u[i] = 0;
-      } else if (a == -2) {
+      const int m[3] = {(c & 1023) + sel, (c >> 10) & 1023, c >> 20};
+      if (from_zero) u[i ^ 1] = 0;
+      if (a == -2) {
         u[i] = 0;
+      } else if constexpr (F64) {
+        const T* row = tb + a * SR;
+        const T s = from_zero ? (T)0 : tail_offdiag64<DIM>(L.n, row, u, i, m);
+        u[i] = (f[i] - s) * row[SR - 1];
       } else {
         const T s = from_zero ? (T)0 : tail_offdiag<T, DIM>(L, tb, u, i, m, a);
         if (a == -1) u[i] = (f[i] - s) * L.inv_dreg;
@@ -472,6 +582,7 @@ __device__ __forceinline__ void vcycle_tail_body(const TailParams<T>& P, const d
   // pre-smoothing of level k (the first sweep from u = 0 when zero) and the restriction
   // of its residual to level k + 1
   auto down = [&](int k, bool zero) {
+    if (G.rank != 0) return;
     for (int it = 0; it < P.nu1; ++it) {
       sweep(k, 0, zero && it == 0);
       sweep(k, 1, false);
@@ -484,6 +595,24 @@ __device__ __forceinline__ void vcycle_tail_body(const TailParams<T>& P, const d
     const int* auxc = sa + P.off[k + 1];
     const T* tb = table(k);
     const T wch = DIM > 2 ? (T)0.125 : (T)0.25;
+    if constexpr (F64) {
+      // a thread per node; the colour that a sweep has just solved for has none (its rounding errors)
+      const int half = (int)L.N / 2;
+      for (int e = tid; e < (P.nu1 > 0 ? half : 2 * half); e += nt) {
+        const int p = e < half ? e : e - half, c = sco[P.off[k] + 2 * p];
+        const int sel = (c + (c >> 10) + (c >> 20) + (e < half ? 0 : 1)) & 1, i = 2 * p + sel;
+        const int a = aux[i];
+        const int m[3] = {(c & 1023) + sel, (c >> 10) & 1023, c >> 20};
+        T r = 0;
+        if (a != -2) {
+          const T* row = tb + a * SR;
+          r = f[i] - fma(row[0], u[i], tail_offdiag64<DIM>(L.n, row, u, i, m));
+        }
+        sr[i] = r;
+        if (P.nu1 > 0) sr[i ^ 1] = 0;
+      }
+      __syncthreads();
+    }
     NodeWalk<DIM> w(C.n, tid, nt);
     for (int I = tid; I < C.N; I += nt, w.advance()) {
       T acc = 0;
@@ -492,10 +621,14 @@ __device__ __forceinline__ void vcycle_tail_body(const TailParams<T>& P, const d
         for (int c = 0; c < nch; ++c) {
           const int m[3] = {2 * w.i0 + (c & 1), 2 * w.i1 + ((c >> 1) & 1), DIM > 2 ? 2 * w.i2 + ((c >> 2) & 1) : 0};
           const int i = m[0] + L.n * (m[1] + L.n * m[2]);
-          const int a = aux[i];
-          if (a == -2) continue;
-          const T dg = a == -1 ? L.dreg : tabd(tb, DIM, a, 0);
-          acc += f[i] - (dg * u[i] + tail_offdiag<T, DIM>(L, tb, u, i, m, a));
+          if constexpr (F64) {
+            acc += sr[i];
+          } else {
+            const int a = aux[i];
+            if (a == -2) continue;
+            const T dg = a == -1 ? L.dreg : tabd(tb, DIM, a, 0);
+            acc += f[i] - (dg * u[i] + tail_offdiag<T, DIM>(L, tb, u, i, m, a));
+          }
         }
         acc *= wch;
       }
@@ -503,30 +636,45 @@ __device__ __forceinline__ void vcycle_tail_body(const TailParams<T>& P, const d
     }
     __syncthreads();
   };
-  // the dense solve on the coarsest level (it does not depend on a starting u)
+  // the dense solve on the coarsest level (it does not depend on a starting u), four rows per warp at
+  // a time: f is gathered once for them, their reads of the inverse are in flight together
   auto coarse = [&]() {
     const int k = P.nlev - 1;
     const LevelK<T>& L = P.L[k];
     T* u = su + P.off[k];
     const T* f = sf + P.off[k];
-    for (int i = tid; i < L.N; i += nt) u[i] = 0;
-    __syncthreads();
+    if (G.rank == 0)
+      for (int i = tid; i < L.N; i += nt) u[i] = 0;
+    G.sync();
     const int lane = tid & 31, wid = tid >> 5, nw = nt / 32;
     int nu = *P.nu_dev;                       // unknowns; the augmentation (if any) follows them
     if (nu < 0 || nu + P.aug > P.ld) {        // a count the dense system has no room for
-      if (tid == 0 && P.status) set_status(P.status, IIM_ERR_CAPACITY);
+      if (G.rank == 0 && tid == 0 && P.status) set_status(P.status, IIM_ERR_CAPACITY);
       nu = 0;
     }
-    for (int r = wid; r < nu; r += nw) {
-      T s = 0;
-      for (int c = lane; c < nu; c += 32) s += P.inv[(size_t)r * P.ld + c] * f[P.map[c]];
-      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      if (lane == 0) u[P.map[r]] = s;
+    if (CLUSTER) {                            // every CTA's own copy: one trip to the first CTA's memory
+      for (int c = tid; c < nu; c += nt) sg[c] = G.load(f + P.map[c]);
+      __syncthreads();
     }
-    __syncthreads();
+    for (int r = 4 * (wid * G.size + G.rank); r < nu; r += 4 * nw * G.size) {
+      T acc[4] = {0, 0, 0, 0};
+      const T* inv = P.inv + (size_t)r * P.ld;
+#pragma unroll 4
+      for (int c = lane; c < nu; c += 32) {
+        const T fv = CLUSTER ? sg[c] : f[P.map[c]];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (r + q < nu) acc[q] += inv[(size_t)q * P.ld + c] * fv;
+      }
+      const T sum = lane_sum4(acc, lane);
+      const int row = r + (lane >> 3);
+      if ((lane & 7) == 0 && row < nu) G.store(u + P.map[row], sum);
+    }
+    G.sync();
   };
   // level k += prolongated correction of level k + 1, then post-smoothing
   auto up = [&](int k) {
+    if (G.rank != 0) return;
     const LevelK<T>& L = P.L[k];
     const LevelK<T>& C = P.L[k + 1];
     T* u = su + P.off[k];
@@ -559,7 +707,10 @@ __device__ __forceinline__ void vcycle_tail_body(const TailParams<T>& P, const d
         if (P.neumann) { acc += ec[ci]; ++cnt; }
         else acc += wgt * ec[ci];
       }
-      if (P.neumann) acc = cnt > 0 ? acc / (T)cnt : (T)0;
+      if (P.neumann) {
+        if constexpr (F64) acc *= cnt > 0 ? kTailInv[cnt] : 0.0;
+        else acc = cnt > 0 ? acc / (T)cnt : (T)0;
+      }
       u[i] += acc;
     }
     __syncthreads();
@@ -613,6 +764,7 @@ __device__ __forceinline__ void vcycle_tail_body(const TailParams<T>& P, const d
       ++cnt[k];
     }
   }
+  if (G.rank != 0) return;
   const LevelK<T>& L = P.L[0];
   for (int i = tid; i < L.N; i += nt) {
     const T u = su[i];
@@ -621,9 +773,9 @@ __device__ __forceinline__ void vcycle_tail_body(const TailParams<T>& P, const d
   }
 }
 
-template <typename T, int DIM>
+template <typename T, int DIM, bool CLUSTER>
 __global__ void __launch_bounds__(kTailThreads) k_vcycle_tail(TailParams<T> P) {
-  vcycle_tail_body<T, DIM>(P, P.v, P.vscale, P.z);
+  vcycle_tail_body<T, DIM, CLUSTER>(P, P.v, P.vscale, P.z);
 }
 
 }  // namespace iim

@@ -496,10 +496,13 @@ TailParams<T> make_tail_params(Problem& P, size_t l0, T* u_out, size_t smem_limi
     tp.toff[k] = toff;
     tp.tcount[k] = P.d_counts + 2 + (int)(l0 + k);
     tp.tcap[k] = L.irr_cap;
-    toff += L.irr_cap * sw_row(L.g.dim);
+    // (the coarsest level's matrix is used in the dense inverse only; FP64: one more row, regular nodes)
+    if (k + 1 < tp.nlev) toff += (L.irr_cap + (sizeof(T) == 8 ? 1 : 0)) * tail_row<T>(L.g.dim);
   }
   tp.toff[tp.nlev] = toff;
-  const size_t base = (sizeof(T) * 2 + 2 * sizeof(int)) * (size_t)off;   // u, f, aux, node coordinates
+  // u, f, aux, node coordinates; FP64: residuals of the largest level
+  const size_t base = (sizeof(T) * 2 + 2 * sizeof(int)) * (size_t)off +
+                      (sizeof(T) == 8 && tp.nlev > 1 ? sizeof(T) * (size_t)tp.off[1] : 0);
   tp.stage_tables = base + sizeof(T) * (size_t)toff <= smem_limit;
   if (!tp.stage_tables) {
     toff = 0;
@@ -539,12 +542,37 @@ static void launch_tail(Problem& P, size_t l0, const double* v, const double* vs
   tp.v = v;
   tp.vscale = vscale;
   tp.z = z;
+  // A dense inverse too large for one SM to read or (FP64) to multiply in a few us is split over a
+  // cluster of eight, whose two barriers cost 1.5 us.  Tail alone / in a cluster, us, by the coarsest
+  // level's nodes: FP32 64: 17.9 / 19.4, 144: 11.8 / 12.7, 196: 13.1 / 13.0, 289: 6.9 / 5.8, 529:
+  // 11.3 / 6.6; FP64 64: 27.1 / 29.2, 100: 14.9 / 15.0, 121: 19.5 / 17.1, 289: 27.1 / 8.8, 529: 57.9 / 11.9.
+  const bool cluster = P.coarse_n >= (sizeof(T) == 8 ? 100 : 200);
+  if (cluster) smem += sizeof(T) * (size_t)P.coarse_n;
+  auto run = [&](auto kernel) {
+    if (smem > 48 * 1024) smem_optin((const void*)kernel);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(cluster ? kTailCluster : 1);
+    cfg.blockDim = dim3(kTailThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = kTailCluster;
+    at[1].val.clusterDim.y = 1;
+    at[1].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = cluster ? 2 : 1;
+    cudaLaunchKernelEx(&cfg, kernel, tp);
+    note_launch();
+  };
   if (P.g.dim == 2) {
-    if (smem > 48 * 1024) smem_optin((const void*)k_vcycle_tail<T, 2>);
-    IIM_LAUNCH_PDL((k_vcycle_tail<T, 2>), 1, kTailThreads, smem, s, tp);
+    if (cluster) run(k_vcycle_tail<T, 2, true>);
+    else run(k_vcycle_tail<T, 2, false>);
   } else {
-    if (smem > 48 * 1024) smem_optin((const void*)k_vcycle_tail<T, 3>);
-    IIM_LAUNCH_PDL((k_vcycle_tail<T, 3>), 1, kTailThreads, smem, s, tp);
+    if (cluster) run(k_vcycle_tail<T, 3, true>);
+    else run(k_vcycle_tail<T, 3, false>);
   }
 }
 
