@@ -400,24 +400,55 @@ __device__ inline bool phase_plus_at(const Geom& G, const double* x) {
   return geom_phi(G, x) >= 0.0;
 }
 
-// Root of phi on the edge [x0, x0 + h e_ax]: safeguarded Newton with bisection.
-// Returns t in [0,1] (fraction of h from x0).  Stops when the bracket or the
+// g and its derivative along axis ax at once: the radius and the angle of a star or a Fourier curve, a
+// dozen FP64 operations each, serve both
+__device__ inline double geom_g_slope(const Geom& G, const double* x, int ax, double* slope) {
+  const double* p = G.p;
+  if (G.kind == IIM_GEOM_STAR || G.kind == IIM_GEOM_FOURIER || G.kind == IIM_GEOM_CIRCLE) {
+    const double dx = x[0] - p[0], dy = x[1] - p[1];
+    const double rho = hypot(dx, dy), ir = 1.0 / rho;
+    double r = p[2], rp = 0.0;
+    if (G.kind != IIM_GEOM_CIRCLE) {
+      const double th = atan2(dy, dx);
+      if (G.kind == IIM_GEOM_STAR) {
+        double sn, cs;
+        sincos(p[4] * th + p[5], &sn, &cs);
+        r = p[2] + p[3] * sn;
+        rp = p[3] * p[4] * cs;
+      } else {
+        double r2;
+        fourier_r(G, th, &r, &rp, &r2);
+      }
+    }
+    const double u = dx * ir, v = dy * ir, q = rp * ir;
+    *slope = ax == 0 ? fma(q, v, u) : fma(-q, u, v);
+    return rho - r;
+  }
+  double gr[3] = {0, 0, 0};
+  geom_grad_g(G, x, gr);
+  *slope = ax == 0 ? gr[0] : (ax == 1 ? gr[1] : gr[2]);
+  return geom_g(G, x);
+}
+
+// Root of phi on the edge [x0, x0 + h e_ax]: safeguarded Newton with bisection; s_lo: x0 is in
+// Omega+ (its phase).  Returns t in [0,1] (fraction of h from x0).  Stops when the bracket or the
 // Newton step is below 2 ulps of 1, i.e. at double precision.
-__device__ inline double edge_root(const Geom& G, const double* x0, int ax, double h, int dim) {
+__device__ inline double edge_root(const Geom& G, const double* x0, int ax, double h, int dim, bool s_lo) {
   double x[3] = {x0[0], x0[1], dim > 2 ? x0[2] : 0.0};
   double lo = 0.0, hi = 1.0;
-  bool s_lo = geom_phi(G, x) >= 0.0;
   double t = 0.5;
   for (int it = 0; it < 100; ++it) {
-    x[ax] = x0[ax] + t * h;
-    double f = geom_phi(G, x);
+    const double xa = (ax == 0 ? x0[0] : (ax == 1 ? x0[1] : x0[2])) + t * h;
+    if (ax == 0) x[0] = xa;
+    else if (ax == 1) x[1] = xa;
+    else x[2] = xa;
+    double slope;
+    const double f = G.sign * geom_g_slope(G, x, ax, &slope);
     if (f == 0.0) break;
     bool s = f >= 0.0;
     if (s == s_lo) lo = t; else hi = t;
     if (hi - lo <= 4.5e-16) break;
-    double gr[3];
-    geom_grad_g(G, x, gr);
-    double df = G.sign * gr[ax] * h;
+    double df = G.sign * slope * h;
     double tn = (df != 0.0) ? t - f / df : 0.5 * (lo + hi);
     if (!(tn > lo && tn < hi)) tn = 0.5 * (lo + hi);
     double step = fabs(tn - t);

@@ -67,7 +67,7 @@ __global__ void k_crossings(Geom G, GridView g, const int32_t* __restrict__ edge
   int m[3];
   node_index(g, i, m);
   double x0[3] = {node_x(g, m[0]), node_x(g, m[1]), g.dim > 2 ? node_x(g, m[2]) : 0.0};
-  double t = edge_root(G, x0, ax, g.h, g.dim);
+  double t = edge_root(G, x0, ax, g.h, g.dim, phase[i] != 0);
   double x[3] = {x0[0], x0[1], x0[2]};
   x[ax] += t * g.h;
   double gr[3] = {0, 0, 0};
@@ -514,7 +514,7 @@ __device__ inline void sw_side(const SWParams& P, const uint8_t* phase, int64_t 
     t = P.cr_t[c];                     // the same root k_crossings found on this edge
   } else {
     double x0[3] = {node_x(g, ml[0]), node_x(g, ml[1]), g.dim > 2 ? node_x(g, ml[2]) : 0.0};
-    t = edge_root(P.G, x0, ax, g.h, g.dim);
+    t = edge_root(P.G, x0, ax, g.h, g.dim, phase[lower] != 0);
   }
   double dist = s > 0 ? t : 1.0 - t;
   kind = P.bc == IIM_BC_DIRICHLET ? S_DIR : S_NEU;
@@ -549,63 +549,92 @@ __global__ void k_sw_classify(SWParams P, const uint8_t* __restrict__ phase, int
   flag[i] = f;
 }
 
-// one thread per irregular node (compacted), so that the FP64 root solves run on full warps
-__global__ void k_sw_fill(SWParams P, const uint8_t* __restrict__ phase, const int32_t* __restrict__ list,
-                          const int* __restrict__ count, int cap, int32_t* __restrict__ aux, double* tab64,
-                          float* tab32, int* status) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
+// Rows of the irregular nodes (compacted) of every level in one launch (blockIdx.y: the level): a lane per
+// side, 4 (2D) or 8 (3D, two idle) per node.  A side's root is a serial chain of FP64 functions, and a
+// warp of whole nodes ran one chain after another for the sides its lanes have cut, 244 us on each of
+// the six levels of a 736^2 star; so did the levels.  The star's set-up takes 1.36 ms for 2.71, that of
+// a 192^3 ellipsoid 10.5 for 11.2.
+struct SWFill {
+  SWParams P;
+  const uint8_t* phase;
+  const int32_t* list;
+  const int* count;
+  int cap;
+  int32_t* aux;
+  double* tab64;
+  float* tab32;
+};
+constexpr int kFillLevels = 12;          // levels per launch (6 KB of arguments)
+struct SWFills {
+  SWFill L[kFillLevels];
+};
+
+__global__ void __launch_bounds__(32) k_sw_fill(const __grid_constant__ SWFills A, int* status) {
+  const SWFill& F = A.L[blockIdx.y];
+  const SWParams& P = F.P;
   const GridView& g = P.g;
-  if (r >= *count || r >= cap) return;
-  const int64_t i = list[r];
-  int m[3];
-  node_index(g, i, m);
-  const int D = sw_row(g.dim);
+  const int dim = g.dim, lanes = dim == 2 ? 4 : 8;
+  const int count = min(*F.count, F.cap);
+  const int first = blockIdx.x * (32 / lanes);
+  if (first >= count) return;
+  const int r = first + (int)threadIdx.x / lanes, k = threadIdx.x % lanes, ax = k >> 1;
+  const bool live = r < count && ax < dim;
+  int64_t i = 0;
+  int kind = S_REG;
+  double psi = 1.0;
+  if (live) {
+    i = F.list[r];
+    int m[3];
+    node_index(g, i, m);
+    sw_side(P, F.phase, i, m, ax, k & 1 ? 1 : -1, kind, psi, status);
+  }
+  const int ko = __shfl_xor_sync(0xffffffffu, kind, 1);
+  const double po = __shfl_xor_sync(0xffffffffu, psi, 1);
+  const int kl = k & 1 ? ko : kind, kr = k & 1 ? kind : ko;
+  const double pl = k & 1 ? po : psi, pr = k & 1 ? psi : po;
+  const int D = sw_row(dim);
   const double h2 = g.h * g.h;
   // interface wall weights (homogeneous Eq. 21, psi = 1/2): uw = lam_m u(minus node) + lam_p u(plus node)
   const double am = 0.5 / P.beta_m, ap = 0.5 / P.beta_p;
   const double lam_minus = ap / (ap + am), lam_plus = am / (ap + am);
-  const bool self_plus = phase[i] != 0;
+  const bool self_plus = live && F.phase[i] != 0;
   const double lam_self = self_plus ? lam_plus : lam_minus, lam_other = self_plus ? lam_minus : lam_plus;
-  double diag = 0, off[6];
-  for (int ax = 0; ax < g.dim; ++ax) {
-    int kl, kr;
-    double pl, pr;
-    sw_side(P, phase, i, m, ax, -1, kl, pl, status);
-    sw_side(P, phase, i, m, ax, +1, kr, pr, status);
-    bool nl = kl == S_NEU, nr = kr == S_NEU;
-    double cl = 0, c0 = 0, cr = 0;
-    if (!nl && !nr) {                       // Eq. 18 (Dirichlet form)
-      cl = 2.0 / (pl * (pl + pr)) / h2;
-      c0 = -2.0 / (pl * pr) / h2;
-      cr = 2.0 / (pr * (pl + pr)) / h2;
-    } else if (nl && !nr) {                 // Eq. 19a
-      c0 = -2.0 / (pr * (2 * pl + pr)) / h2;
-      cr = 2.0 / (pr * (2 * pl + pr)) / h2;
-    } else if (nr && !nl) {                 // Eq. 19b (psi- in the denominators)
-      cl = 2.0 / (pl * (pl + 2 * pr)) / h2;
-      c0 = -2.0 / (pl * (pl + 2 * pr)) / h2;
-    }
-    diag += c0;
-    double ol = 0, orr = 0;
-    if (kl == S_REG) ol = cl;
-    else if (kl == S_IF) { diag += cl * lam_self; ol = cl * lam_other; }
-    if (kr == S_REG) orr = cr;
-    else if (kr == S_IF) { diag += cr * lam_self; orr = cr * lam_other; }
-    off[2 * ax] = ol;
-    off[2 * ax + 1] = orr;
+  const bool nl = kl == S_NEU, nr = kr == S_NEU;
+  double cl = 0, c0 = 0, cr = 0;
+  if (!nl && !nr) {                       // Eq. 18 (Dirichlet form)
+    cl = 2.0 / (pl * (pl + pr)) / h2;
+    c0 = -2.0 / (pl * pr) / h2;
+    cr = 2.0 / (pr * (pl + pr)) / h2;
+  } else if (nl && !nr) {                 // Eq. 19a
+    c0 = -2.0 / (pr * (2 * pl + pr)) / h2;
+    cr = 2.0 / (pr * (2 * pl + pr)) / h2;
+  } else if (nr && !nl) {                 // Eq. 19b (psi- in the denominators)
+    cl = 2.0 / (pl * (pl + 2 * pr)) / h2;
+    c0 = -2.0 / (pl * (pl + 2 * pr)) / h2;
   }
-  tab64[(size_t)r * D] = diag;
-  tab32[(size_t)r * D] = (float)diag;
-  for (int k = 0; k < 2 * g.dim; ++k) {
-    tab64[(size_t)r * D + 1 + k] = off[k];
-    tab32[(size_t)r * D + 1 + k] = (float)off[k];
+  // the diagonal over the axes in order, in the first lane
+  double diag = 0;
+  for (int a = 0; a < dim; ++a) {
+    const int from = ((int)threadIdx.x / lanes) * lanes + 2 * a;
+    diag += __shfl_sync(0xffffffffu, c0, from);
+    const double vl = __shfl_sync(0xffffffffu, cl, from), vr = __shfl_sync(0xffffffffu, cr, from);
+    if (__shfl_sync(0xffffffffu, kl, from) == S_IF) diag += vl * lam_self;
+    if (__shfl_sync(0xffffffffu, kr, from) == S_IF) diag += vr * lam_self;
   }
-  if (g.dim > 2) {                       // 3D rows carry the reciprocal diagonal in their last entry
+  if (!live) return;
+  const double c = k & 1 ? cr : cl;
+  const double off = kind == S_REG ? c : (kind == S_IF ? c * lam_other : 0.0);
+  F.tab64[(size_t)r * D + 1 + k] = off;
+  F.tab32[(size_t)r * D + 1 + k] = (float)off;
+  if (k != 0) return;
+  F.tab64[(size_t)r * D] = diag;
+  F.tab32[(size_t)r * D] = (float)diag;
+  if (dim > 2) {                         // 3D rows carry the reciprocal diagonal in their last entry
     const double inv = diag != 0.0 ? 1.0 / diag : 0.0;
-    tab64[(size_t)r * D + 7] = inv;
-    tab32[(size_t)r * D + 7] = (float)inv;
+    F.tab64[(size_t)r * D + 7] = inv;
+    F.tab32[(size_t)r * D + 7] = (float)inv;
   }
-  aux[i] = r;
+  F.aux[i] = r;
 }
 
 // outer-box sample points: face f = 2 ax + (side > 0), then the other node indices of the
@@ -742,6 +771,14 @@ iim_status setup_fits(Problem& P) {
 
 iim_status setup_levels(Problem& P, bool size_only) {
   const int T = 256;
+  SWFills fills;
+  int held = 0, most = 0;                // levels in fills, and the largest capacity among them
+  auto fill = [&]() {
+    if (held == 0) return;
+    const int per = P.g.dim == 2 ? 8 : 4;
+    IIM_LAUNCH(k_sw_fill, dim3(ceil_div(most, per), held), 32, 0, P.stream, fills, P.d_status);
+    held = most = 0;
+  };
   for (size_t l = 0; l < P.lv.size(); ++l) {
     Level& L = P.lv[l];
     SWParams S{L.g, P.geom, P.desc.bc == IIM_BC_INTERFACE, P.desc.bc, P.desc.box_bc, P.desc.beta_plus,
@@ -757,9 +794,11 @@ iim_status setup_levels(Problem& P, bool size_only) {
     if (size_only) continue;
     IIM_LAUNCH(k_compact, ceil_div(L.g.N, T), T, 0, P.stream, L.flag, L.idx, L.g.N, L.irr_cap, L.irr_node,
                P.d_status);
-    IIM_LAUNCH(k_sw_fill, ceil_div(L.irr_cap, 32), 32, 0, P.stream, S, L.phase, L.irr_node, P.d_counts + 2 + (int)l,
-               L.irr_cap, L.aux, L.tab64, L.tab32, P.d_status);
+    fills.L[held++] = SWFill{S, L.phase, L.irr_node, P.d_counts + 2 + (int)l, L.irr_cap, L.aux, L.tab64, L.tab32};
+    most = std::max(most, L.irr_cap);
+    if (held == kFillLevels) fill();
   }
+  fill();
   return IIM_OK;
 }
 
