@@ -13,7 +13,7 @@
 //   MODE 6  MODE 2 and MODE 3 in one kernel (nu2 = 2)
 //   MODE 7  MODE 5 from a given u (a W-cycle's second visit of a level): halo 5, since
 //           the first half sweep now reads its neighbours
-// Coarse tail: every level with at most 1024 nodes (one per thread) and the dense
+// Coarse tail: every level with at most 1024 nodes (a pair per thread) and the dense
 // coarse solve run in a single CTA with the whole sub-hierarchy in shared memory.
 #pragma once
 
@@ -328,7 +328,8 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 7 : 1) k_mg2d(Fine2DPara
 constexpr int kTailMaxLevels = 8;
 constexpr int kTailNodes = 1024;      // levels with at most this many nodes go to the tail
 constexpr int kTailCluster = 8;       // CTAs that share a large dense solve
-constexpr int kTailThreads = 1024;    // threads of the tail's CTA: one node each on its first level
+constexpr int kTailThreads = 512;     // threads of the tail's CTA: a pair of nodes each on its first level
+static_assert(kTailNodes <= 2 * kTailThreads, "a pair of nodes per thread");
 
 template <typename T>
 struct TailParams {
@@ -381,34 +382,12 @@ __device__ inline T tail_offdiag(const LevelK<T>& L, const T* tb, const T* u, in
   return s;
 }
 
-// node -> (i0, i1, i2) for the nodes i = t, t + stride, ...: one division per level, then
-// a carry per step (stride is the block size)
-template <int DIM>
-struct NodeWalk {
-  int n, i0, i1, i2, d0, drow;
-  __device__ NodeWalk(int n_, int start, int stride) : n(n_) {
-    i0 = start % n;
-    const int r = start / n;
-    i1 = DIM > 2 ? r % n : r;
-    i2 = DIM > 2 ? r / n : 0;
-    d0 = stride % n;
-    drow = stride / n;
-  }
-  __device__ void advance() {
-    i0 += d0;
-    int rows = drow;
-    if (i0 >= n) { i0 -= n; ++rows; }
-    i1 += rows;
-    if (DIM > 2 && i1 >= n) { i2 += i1 / n; i1 %= n; }
-  }
-};
-
 // FP64 tails stage their rows as [diagonal, off-diagonals, 1 / diagonal], with one more for the regular
 // nodes, so that every node of a sweep runs the same few FP64 operations: a division takes the place of
 // a dozen, and one irregular node makes its whole warp run the second path (GB300 issues two FP64
 // operations per clock and SM, and the tail has one to a few SMs).  With that, full warps per colour and
-// the shared dense solve the tail of a 104^2 problem (26^2, 13^2) takes 19.6 us for 71.0, of a 120^2 one
-// 23.3 for 94.8, of 40^3 30.6 for 121; FP32, same arithmetic as before, 12.6 for 14.5 and 13.1 for 16.7.
+// the shared dense solve the tail of a 104^2 problem (26^2, 13^2) takes 16.5 us for 71.0, of a 120^2 one
+// 20.0 for 94.8, of 40^3 29.1 for 121; FP32, same arithmetic as before, 11.3 for 14.5 and 11.6 for 16.7.
 __host__ __device__ constexpr int tail_row64(int dim) { return 2 * dim + 2; }
 template <typename T>
 __host__ __device__ constexpr int tail_row(int dim) { return sizeof(T) == 8 ? tail_row64(dim) : sw_row(dim); }
@@ -548,33 +527,53 @@ __device__ __forceinline__ void vcycle_tail_body(const TailParams<T>& P, const d
     }
     __syncthreads();
   }
-  // A thread takes a node of every second, 2 p or 2 p + 1 by colour (the levels that are smoothed have
-  // been halved, so their rows are even): full warps, where one thread per node left half of each idle.
-  auto sweep = [&](int k, int colour, bool from_zero) {
+  // the relaxed value of node i (coordinates m, class a, right-hand side f)
+  auto relaxed = [&](const LevelK<T>& L, const T* tb, const T* u, int i, const int* m, int a, T f, bool from_zero) -> T {
+    if (a == -2) return 0;
+    if constexpr (F64) {
+      const T* row = tb + a * SR;
+      const T s = from_zero ? (T)0 : tail_offdiag64<DIM>(L.n, row, u, i, m);
+      return (f - s) * row[SR - 1];
+    } else {
+      const T s = from_zero ? (T)0 : tail_offdiag<T, DIM>(L, tb, u, i, m, a);
+      if (a == -1) return (f - s) * L.inv_dreg;
+      const T dg = tabd(tb, DIM, a, 0);
+      return dg != (T)0 ? (f - s) / dg : (T)0;
+    }
+  };
+  // `its` sweeps of both colours on level k (the first from u = 0 when zero).  A thread owns nodes 2 p and
+  // 2 p + 1, one of each colour (the levels that are smoothed have been halved, so their rows are even):
+  // full warps, and what does not change from sweep to sweep stays in registers.  Only the warps that own
+  // nodes meet between the half sweeps; that meeting is most of a small level's time.  512 threads, for
+  // 1024 that each looked up a node per half sweep: 32^2, 16^2 and 8^2 in 14.5 us for 17.9, 8^3 and 4^3 in
+  // 10.0 for 13.5, the same bits.
+  auto smooth = [&](int k, int its, bool zero) {
     const LevelK<T>& L = P.L[k];
     T* u = su + P.off[k];
-    const T* f = sf + P.off[k];
     const T* tb = table(k);
-    const int half = (int)L.N / 2;
-    for (int p = tid; p < half; p += nt) {
-      const int c = sco[P.off[k] + 2 * p];
-      const int sel = (c + (c >> 10) + (c >> 20) + colour) & 1, i = 2 * p + sel;
-      const int a = sa[P.off[k] + i];
-      const int m[3] = {(c & 1023) + sel, (c >> 10) & 1023, c >> 20};
-      if (from_zero) u[i ^ 1] = 0;
-      if (a == -2) {
-        u[i] = 0;
-      } else if constexpr (F64) {
-        const T* row = tb + a * SR;
-        const T s = from_zero ? (T)0 : tail_offdiag64<DIM>(L.n, row, u, i, m);
-        u[i] = (f[i] - s) * row[SR - 1];
-      } else {
-        const T s = from_zero ? (T)0 : tail_offdiag<T, DIM>(L, tb, u, i, m, a);
-        if (a == -1) u[i] = (f[i] - s) * L.inv_dreg;
-        else {
-          const T dg = tabd(tb, DIM, a, 0);
-          u[i] = dg != (T)0 ? (f[i] - s) / dg : (T)0;
+    const int warps = ((int)L.N / 2 + 31) >> 5;
+    if ((tid >> 5) < warps && its > 0) {
+      const bool live = tid < (int)L.N / 2;
+      const int p = live ? tid : 0, c = sco[P.off[k] + 2 * p];
+      const int red = (c + (c >> 10) + (c >> 20)) & 1;
+      const int i0 = 2 * p + red, i1 = 2 * p + 1 - red;
+      const int m0[3] = {(c & 1023) + red, (c >> 10) & 1023, c >> 20};
+      const int m1[3] = {(c & 1023) + 1 - red, m0[1], m0[2]};
+      const int a0 = sa[P.off[k] + i0], a1 = sa[P.off[k] + i1];
+      const T f0 = sf[P.off[k] + i0], f1 = sf[P.off[k] + i1];
+      auto meet = [&]() {
+        if (warps == 1) __syncwarp();
+        else asm volatile("bar.sync 1, %0;" ::"r"(warps * 32) : "memory");
+      };
+      for (int it = 0; it < its; ++it) {
+        const bool fz = zero && it == 0;
+        if (live) {
+          if (fz) u[i1] = 0;
+          u[i0] = relaxed(L, tb, u, i0, m0, a0, f0, fz);
         }
+        meet();
+        if (live) u[i1] = relaxed(L, tb, u, i1, m1, a1, f1, false);
+        meet();
       }
     }
     __syncthreads();
@@ -583,10 +582,7 @@ __device__ __forceinline__ void vcycle_tail_body(const TailParams<T>& P, const d
   // of its residual to level k + 1
   auto down = [&](int k, bool zero) {
     if (G.rank != 0) return;
-    for (int it = 0; it < P.nu1; ++it) {
-      sweep(k, 0, zero && it == 0);
-      sweep(k, 1, false);
-    }
+    smooth(k, P.nu1, zero);
     const LevelK<T>& L = P.L[k];
     const LevelK<T>& C = P.L[k + 1];
     const T* u = su + P.off[k];
@@ -613,26 +609,40 @@ __device__ __forceinline__ void vcycle_tail_body(const TailParams<T>& P, const d
       }
       __syncthreads();
     }
-    NodeWalk<DIM> w(C.n, tid, nt);
-    for (int I = tid; I < C.N; I += nt, w.advance()) {
-      T acc = 0;
-      if (auxc[I] != -2) {
-        constexpr int nch = 1 << DIM;
-        for (int c = 0; c < nch; ++c) {
-          const int m[3] = {2 * w.i0 + (c & 1), 2 * w.i1 + ((c >> 1) & 1), DIM > 2 ? 2 * w.i2 + ((c >> 2) & 1) : 0};
+    constexpr int nch = 1 << DIM;
+    if constexpr (F64) {
+      for (int I = tid; I < C.N; I += nt) {
+        T acc = 0;
+        if (auxc[I] != -2) {
+          const int cc = sco[P.off[k + 1] + I];
+          const int i = 2 * (cc & 1023) + L.n * (2 * ((cc >> 10) & 1023) + L.n * 2 * (cc >> 20));
+#pragma unroll
+          for (int c = 0; c < nch; ++c) acc += sr[i + (c & 1) + L.n * (((c >> 1) & 1) + L.n * (c >> 2))];
+          acc *= wch;
+        }
+        sf[P.off[k + 1] + I] = store_residual(acc, C.f_bf16);
+      }
+    } else {
+      // a lane per child, added in their order
+      const int lane = tid & 31, total = (int)C.N * nch;
+      for (int base = tid - lane; base < total; base += nt) {
+        const int e = base + lane, I = e / nch, c = e % nch;
+        T r = 0;
+        if (e < total && auxc[I] != -2) {
+          const int cc = sco[P.off[k + 1] + I];
+          const int m[3] = {2 * (cc & 1023) + (c & 1), 2 * ((cc >> 10) & 1023) + ((c >> 1) & 1), 2 * (cc >> 20) + (c >> 2)};
           const int i = m[0] + L.n * (m[1] + L.n * m[2]);
-          if constexpr (F64) {
-            acc += sr[i];
-          } else {
-            const int a = aux[i];
-            if (a == -2) continue;
+          const int a = aux[i];
+          if (a != -2) {
             const T dg = a == -1 ? L.dreg : tabd(tb, DIM, a, 0);
-            acc += f[i] - (dg * u[i] + tail_offdiag<T, DIM>(L, tb, u, i, m, a));
+            r = f[i] - (dg * u[i] + tail_offdiag<T, DIM>(L, tb, u, i, m, a));
           }
         }
-        acc *= wch;
+        T acc = 0;
+#pragma unroll
+        for (int q = 0; q < nch; ++q) acc += __shfl_sync(0xffffffffu, r, (lane & ~(nch - 1)) + q);
+        if (e < total && c == 0) sf[P.off[k + 1] + I] = store_residual(acc * wch, C.f_bf16);
       }
-      sf[P.off[k + 1] + I] = store_residual(acc, C.f_bf16);
     }
     __syncthreads();
   };
@@ -681,18 +691,20 @@ __device__ __forceinline__ void vcycle_tail_body(const TailParams<T>& P, const d
     const T* ec = su + P.off[k + 1];
     const int* aux = sa + P.off[k];
     const int* auxc = sa + P.off[k + 1];
-    NodeWalk<DIM> w(L.n, tid, nt);
-    for (int i = tid; i < L.N; i += nt, w.advance()) {
+    for (int i = tid; i < L.N; i += nt) {
       if (aux[i] == -2) continue;
-      const int I[3] = {w.i0 >> 1, w.i1 >> 1, w.i2 >> 1};
-      const int sg[3] = {(w.i0 & 1) ? 1 : -1, (w.i1 & 1) ? 1 : -1, (w.i2 & 1) ? 1 : -1};
+      const int cc = sco[P.off[k] + i], w0 = cc & 1023, w1 = (cc >> 10) & 1023, w2 = cc >> 20;
+      const int I[3] = {w0 >> 1, w1 >> 1, w2 >> 1};
+      const int sg[3] = {(w0 & 1) ? 1 : -1, (w1 & 1) ? 1 : -1, (w2 & 1) ? 1 : -1};
       T acc = 0;
       int cnt = 0;
       constexpr int nsel = 1 << DIM;
+#pragma unroll
       for (int sel = 0; sel < nsel; ++sel) {
         int c[3];
         T wgt = 1;
         bool inb = true;
+#pragma unroll
         for (int q = 0; q < 3; ++q) {
           const int b = (sel >> q) & 1;
           c[q] = q < DIM ? I[q] + b * sg[q] : 0;
@@ -714,10 +726,7 @@ __device__ __forceinline__ void vcycle_tail_body(const TailParams<T>& P, const d
       u[i] += acc;
     }
     __syncthreads();
-    for (int it = 0; it < P.nu2; ++it) {
-      sweep(k, 0, false);
-      sweep(k, 1, false);
-    }
+    smooth(k, P.nu2, false);
   };
   // Visit schedule (Sec. 3.3 results): each visit of level k below the first runs gamma
   // visits of level k + 1, the second from the first one's result with the same f; the
@@ -774,7 +783,7 @@ __device__ __forceinline__ void vcycle_tail_body(const TailParams<T>& P, const d
 }
 
 template <typename T, int DIM, bool CLUSTER>
-__global__ void __launch_bounds__(kTailThreads) k_vcycle_tail(TailParams<T> P) {
+__global__ void __launch_bounds__(kTailThreads, 1) k_vcycle_tail(TailParams<T> P) {
   vcycle_tail_body<T, DIM, CLUSTER>(P, P.v, P.vscale, P.z);
 }
 

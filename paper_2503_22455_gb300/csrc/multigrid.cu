@@ -544,7 +544,7 @@ static void launch_tail(Problem& P, size_t l0, const double* v, const double* vs
   tp.z = z;
   // A dense inverse too large for one SM to read or (FP64) to multiply in a few us is split over a
   // cluster of eight, whose two barriers cost 1.5 us.  Tail alone / in a cluster, us, by the coarsest
-  // level's nodes: FP32 64: 17.9 / 19.4, 144: 11.8 / 12.7, 196: 13.1 / 13.0, 289: 6.9 / 5.8, 529:
+  // level's nodes (with 1024 threads): FP32 64: 17.9 / 19.4, 144: 11.8 / 12.7, 196: 13.1 / 13.0, 289: 6.9 / 5.8, 529:
   // 11.3 / 6.6; FP64 64: 27.1 / 29.2, 100: 14.9 / 15.0, 121: 19.5 / 17.1, 289: 27.1 / 8.8, 529: 57.9 / 11.9.
   const bool cluster = P.coarse_n >= (sizeof(T) == 8 ? 100 : 200);
   if (cluster) smem += sizeof(T) * (size_t)P.coarse_n;
