@@ -13,15 +13,15 @@
 //     cells and for cells at a box face alone, whose weights follow from the position;
 //   - the first half sweep from u = 0 is a product and comes with the entry of f, the last one with
 //     the exit of z;
-//   - a half sweep goes through 16 planes per thread on the levels that exceed L2, so that a plane
-//     crosses L2 once per run instead of three times.
+//   - on the levels that exceed L2 a half sweep goes through several planes per thread, two pairs
+//     at a time, so that a plane crosses L2 once per run instead of three times.
 // Not kept: all four half sweeps in one kernel that streams planes through registers (1.5 ms per
 // cycle at 256^3: 500 dependent instructions per warp and plane), and the natural order of u and f
 // (0.80 ms).
 //
 // Measured (V-cycle, FP32, against one kernel per half sweep in natural order with 64-bit index
-// divisions and 4-byte row codes): 256^3 exterior ellipsoid 2.28 -> 0.78 ms, 96^3 perturbed sphere
-// 0.27 -> 0.10 ms; 128^3 in FP64 0.53 ms.
+// divisions and 4-byte row codes): 256^3 exterior ellipsoid 2.28 -> 0.69 ms, 96^3 perturbed sphere
+// 0.27 -> 0.10 ms; 128^3 in FP64 0.52 ms.
 #pragma once
 
 namespace iim {
@@ -127,47 +127,116 @@ __global__ void __launch_bounds__(256) k_first3d(Grid3D<T> G, const double* __re
   u[q.p] = r;
 }
 
-// One half sweep in place (cells that are no unknowns get 0); OUT: the level's result leaves as FP64
-// (finest level, last half sweep).  A thread goes through `run` planes: the other colour's value at
-// its place in the next plane becomes the x neighbour there and the z neighbour one plane on, so a
-// plane of u crosses L2 once per run instead of three times.
+// One half sweep in place (cells that are no unknowns get 0), a thread per pair; OUT: the level's result
+// leaves as FP64 (finest level, last half sweep).
 template <typename T, bool OUT>
 __global__ void __launch_bounds__(256) k_smooth3d(Grid3D<T> G, T* __restrict__ u, const T* __restrict__ f, int f_bf16,
-                                                  int colour, int run, double* __restrict__ zout) {
-  const int n = G.n, h = n / 2, hn = h * n, half = n * hn;
-  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
-  const int y = (int)(t / (unsigned)h), k = (int)(t - (unsigned)y * (unsigned)h);
-  const int z0 = blockIdx.y * run, z1 = min(n, z0 + run);
+                                                  int colour, double* __restrict__ zout) {
+  const Pair3D q(G.n);
+  const int n = G.n, h = n / 2, hn = h * n, half = n * hn, p = q.p;
   const T* o = u + (colour ? 0 : half);
   T* own = u + (colour ? half : 0);
-  const T* fo = f;
-  const int fofs = colour ? half : 0;
-  const bool in = y < n;
-  int p = z0 * hn + (int)t;
-  uint8_t w = in ? __ldg(G.cls + 2 * p + ((y + z0 + colour) & 1)) : 0;
+  const int e = (q.y + q.z + colour) & 1;
+  const bool in = q.y < n;
+  const uint8_t w = in ? __ldg(G.cls + 2 * p + e) : 0;
   pdl_trigger();
   pdl_wait();
   if (!in) return;
-  T om = z0 > 0 ? o[p - hn] : (T)0, oc = o[p];
+  T val = 0;
+  const T oc = o[p];
+  if (w & kClsUnknown) {
+    const T side = e ? (q.k < h - 1 ? o[p + 1] : (T)0) : (q.k > 0 ? o[p - 1] : (T)0);
+    const T v[6] = {e ? oc : side, e ? side : oc, q.y > 0 ? o[p - h] : (T)0, q.y < n - 1 ? o[p + h] : (T)0,
+                    q.z > 0 ? o[p - hn] : (T)0, q.z < n - 1 ? o[p + hn] : (T)0};
+    T diag, inv;
+    const T r = row_minus(G, 2 * q.k + e, q.y, q.z, w, load_f(f, (colour ? half : 0) + p, f_bf16), v, diag, inv);
+    val = mul_rn(r, inv);
+  }
+  if (OUT) {
+    double2 st;
+    st.x = (double)(e ? oc : val);
+    st.y = (double)(e ? val : oc);
+    *(double2*)(zout + 2 * p) = st;
+  } else {
+    own[p] = val;
+  }
+}
+
+// two consecutive values of one colour
+template <typename T>
+struct Two {
+  T a, b;
+};
+__device__ __forceinline__ Two<float> load_two(const float* p) {
+  const float2 v = *reinterpret_cast<const float2*>(p);
+  return {v.x, v.y};
+}
+__device__ __forceinline__ Two<double> load_two(const double* p) {
+  const double2 v = *reinterpret_cast<const double2*>(p);
+  return {v.x, v.y};
+}
+__device__ __forceinline__ void store_two(float* p, float a, float b) { *reinterpret_cast<float2*>(p) = make_float2(a, b); }
+__device__ __forceinline__ void store_two(double* p, double a, double b) { *reinterpret_cast<double2*>(p) = make_double2(a, b); }
+
+// The same for levels that exceed L2 (n a multiple of 4): a thread takes two neighbouring pairs through
+// `run` planes.  The other colour's values at its places in the next plane become the x neighbours there
+// and the z neighbours one plane on, so a plane of u crosses L2 once per run instead of three times; the
+// pairs share a vector load per neighbour row, the x neighbour between them and the index arithmetic,
+// which bounded the single pairs (99 instructions per cell, 67 % of the issue slots): 41.4 -> 30.1 us per
+// half sweep at 256^3 (17 us for its bytes), V-cycle 777 -> 689 us.
+template <typename T, bool OUT>
+__global__ void __launch_bounds__(256) k_smooth3d_run(Grid3D<T> G, T* __restrict__ u, const T* __restrict__ f,
+                                                      int f_bf16, int colour, int run, double* __restrict__ zout) {
+  const int n = G.n, h = n / 2, hn = h * n, half = n * hn;
+  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
+  const int y = (int)(t / (unsigned)(h / 2)), k = 2 * (int)(t - (unsigned)y * (unsigned)(h / 2));
+  const int z0 = blockIdx.y * run, z1 = min(n, z0 + run);
+  const T* o = u + (colour ? 0 : half);
+  T* own = u + (colour ? half : 0);
+  const int fofs = colour ? half : 0;
+  const bool in = y < n;
+  int p = z0 * hn + y * h + k;
+  // classes of the four cells of both pairs
+  unsigned w = in ? __ldg((const unsigned*)(G.cls + 2 * p)) : 0;
+  pdl_trigger();
+  pdl_wait();
+  if (!in) return;
+  const Two<T> zero = {(T)0, (T)0};
+  Two<T> om = z0 > 0 ? load_two(o + p - hn) : zero, oc = load_two(o + p);
   for (int z = z0; z < z1; ++z, p += hn) {
     const int e = (y + z + colour) & 1;
-    const T op = z < n - 1 ? o[p + hn] : (T)0;
-    const uint8_t wn = z + 1 < z1 ? __ldg(G.cls + 2 * (p + hn) + (e ^ 1)) : 0;
-    T val = 0;
-    if (w & kClsUnknown) {
-      const T side = e ? (k < h - 1 ? o[p + 1] : (T)0) : (k > 0 ? o[p - 1] : (T)0);
-      const T v[6] = {e ? oc : side, e ? side : oc, y > 0 ? o[p - h] : (T)0, y < n - 1 ? o[p + h] : (T)0, om, op};
-      T diag, inv;
-      const T r = row_minus(G, 2 * k + e, y, z, w, load_f(fo, fofs + p, f_bf16), v, diag, inv);
-      val = mul_rn(r, inv);
+    const Two<T> op = z < n - 1 ? load_two(o + p + hn) : zero;
+    const unsigned wn = z + 1 < z1 ? __ldg((const unsigned*)(G.cls + 2 * (p + hn))) : 0;
+    const unsigned wa = (w >> (8 * e)) & 255, wb = (w >> (16 + 8 * e)) & 255;
+    T va = 0, vb = 0;
+    if ((wa | wb) & kClsUnknown) {
+      const T side = e ? (k + 2 < h ? o[p + 2] : (T)0) : (k > 0 ? o[p - 1] : (T)0);
+      const Two<T> ym = y > 0 ? load_two(o + p - h) : zero, yp = y < n - 1 ? load_two(o + p + h) : zero;
+      Two<T> ff;
+      if (f_bf16) ff = {load_f(f, fofs + p, f_bf16), load_f(f, fofs + p + 1, f_bf16)};
+      else ff = load_two(f + fofs + p);
+      const T a[6] = {e ? oc.a : side, e ? oc.b : oc.a, ym.a, yp.a, om.a, op.a};
+      const T b[6] = {e ? oc.b : oc.a, e ? side : oc.b, ym.b, yp.b, om.b, op.b};
+      if ((wa & wb & kClsUnknown) && !((wa | wb) & kClsIrregular)) {
+        va = mul_rn(off_residual3(ff.a, G.ih2, G.ih2, G.ih2, G.ih2, G.ih2, G.ih2, a[0], a[1], a[2], a[3], a[4], a[5]), G.inv_dreg);
+        vb = mul_rn(off_residual3(ff.b, G.ih2, G.ih2, G.ih2, G.ih2, G.ih2, G.ih2, b[0], b[1], b[2], b[3], b[4], b[5]), G.inv_dreg);
+      } else {
+        T diag, inv;
+        if (wa & kClsUnknown) {
+          const T r = row_minus(G, 2 * k + e, y, z, (uint8_t)wa, ff.a, a, diag, inv);
+          va = mul_rn(r, inv);
+        }
+        if (wb & kClsUnknown) {
+          const T r = row_minus(G, 2 * k + 2 + e, y, z, (uint8_t)wb, ff.b, b, diag, inv);
+          vb = mul_rn(r, inv);
+        }
+      }
     }
     if (OUT) {
-      double2 st;
-      st.x = (double)(e ? oc : val);
-      st.y = (double)(e ? val : oc);
-      *(double2*)(zout + 2 * p) = st;
+      *(double2*)(zout + 2 * p) = make_double2((double)(e ? oc.a : va), (double)(e ? va : oc.a));
+      *(double2*)(zout + 2 * p + 2) = make_double2((double)(e ? oc.b : vb), (double)(e ? vb : oc.b));
     } else {
-      own[p] = val;
+      store_two(own + p, va, vb);
     }
     om = oc;
     oc = op;

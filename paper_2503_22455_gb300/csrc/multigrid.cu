@@ -740,10 +740,24 @@ static Grid3D<T> grid3d(const Level& L) {
   return G;
 }
 
-// Planes per thread of a half sweep: 16 on the levels whose u and f take more than half of L2
-// (256^3: 51 -> 41 us per half sweep); one below, where the loop only adds latency (128^3: 9.6 us
-// against 10.7 with runs of 4).
-static int smooth3d_run(int n) { return (int64_t)n * n * n * 8 > (64 << 20) ? 16 : 1; }
+// One half sweep of a 3D level.  Levels whose u and f take more than half of L2 go through 4 planes per
+// thread, two pairs at a time (256^3: V-cycle 689 us; 8 planes 699, 16 planes 765, a pair and 16 planes
+// 777); below, a plane per thread, where the loop only adds latency (V-cycle 192^3 240 us against 249
+// with runs, 128^3 158 / 171, 96^3 101 / 128).
+constexpr int kSmooth3dRun = 4;
+template <typename T>
+static void smooth3d(const Grid3D<T>& G, T* u, const T* f, int f_bf16, int colour, double* z, cudaStream_t s) {
+  const int n = G.n;
+  if ((int64_t)n * n * n * 8 > (64 << 20) && n % 4 == 0) {
+    const dim3 grid(ceil_div((int64_t)n * (n / 4), 256), ceil_div(n, kSmooth3dRun));
+    if (z) IIM_LAUNCH_PDL((k_smooth3d_run<T, true>), grid, 256, 0, s, G, u, f, f_bf16, colour, kSmooth3dRun, z);
+    else IIM_LAUNCH_PDL((k_smooth3d_run<T, false>), grid, 256, 0, s, G, u, f, f_bf16, colour, kSmooth3dRun, z);
+    return;
+  }
+  const dim3 grid(ceil_div((int64_t)n * (n / 2), 256), n);
+  if (z) IIM_LAUNCH_PDL((k_smooth3d<T, true>), grid, 256, 0, s, G, u, f, f_bf16, colour, z);
+  else IIM_LAUNCH_PDL((k_smooth3d<T, false>), grid, 256, 0, s, G, u, f, f_bf16, colour, z);
+}
 
 // 3D: u of every level is updated in place (stored by colour above the tail) and starts from zero unless this is a later visit of a
 // W-cycle.  The level's right-hand side is v scale / beta on the finest level (v set), else L.f; the
@@ -761,11 +775,8 @@ static void vcycle3d(Problem& P, size_t l, size_t lt, const double* v, const dou
   const int Tn = 256, n = L.g.n;
   const Grid3D<T> G = grid3d<T>(L);
   const dim3 grid(ceil_div(n * (n / 2), Tn), n);
-  const int run = smooth3d_run(n);
-  const dim3 grid_s(grid.x, ceil_div(n, run));
   auto sweep = [&](int colour, bool out) {
-    if (out) IIM_LAUNCH_PDL((k_smooth3d<T, true>), grid_s, Tn, 0, s, G, u, (const T*)f, L.f_bf16, colour, run, z);
-    else IIM_LAUNCH_PDL((k_smooth3d<T, false>), grid_s, Tn, 0, s, G, u, (const T*)f, L.f_bf16, colour, run, (double*)nullptr);
+    smooth3d<T>(G, u, (const T*)f, L.f_bf16, colour, out ? z : nullptr, s);
   };
   if (from_zero)
     IIM_LAUNCH_PDL(k_first3d<T>, grid, Tn, 0, s, G, v, vscale, (T)(1.0 / P.desc.beta_plus), (T)(1.0 / P.desc.beta_minus),
@@ -860,10 +871,7 @@ template <typename T>
 static void smooth_fine_t(Problem& P, int colour, cudaStream_t s) {
   Level& L = P.lv[0];
   if (P.g.dim == 3 && tail_start(P) > 0) {
-    const int n = L.g.n;
-    const int run = smooth3d_run(n);
-    IIM_LAUNCH_PDL((k_smooth3d<T, false>), dim3(ceil_div(n * (n / 2), 256), ceil_div(n, run)), 256, 0, s, grid3d<T>(L),
-                   (T*)L.u, (const T*)L.f, L.f_bf16, colour, run, (double*)nullptr);
+    smooth3d<T>(grid3d<T>(L), (T*)L.u, (const T*)L.f, L.f_bf16, colour, nullptr, s);
     return;
   }
   LevelView<T> V = view<T>(L);
