@@ -15,7 +15,7 @@
 // the rest of the grid, so that neither the ghost values nor the corrections add to the time of
 // the plain nodes.  Three kernels, the ghosts on a second stream between two events and the
 // corrections after both, took 17.2 us for a 64^2 circle and 57.5 us for the order-6 star at
-// 1024^2; the two take 9.4 to 12.5 and 43.6.
+// 1024^2; the two take 9.4 to 12.5 and 38.8.
 // The plain nodes are FP64 and bound by the FP64 pipe on GB300 (2 FMA/clk/SM), so they are
 // written to use the fewest FP64 operations: neighbours at equal |j| are summed first, then
 // one FMA per |j| with beta/h^2 folded into the coefficients.  Large 3D grids sum in fixed point
@@ -74,7 +74,7 @@ __device__ __forceinline__ void ho_stencil_node(const GridView& g, const Stencil
 // of every row (sequential FMAs, no per-term reduction), then two shuffle steps
 // combine the quarters.  Boundary problems: rows 0..w-1 of fit c.  Interface
 // problems: rows 0..w of fits 2c (+) and 2c+1 (-), then the closure of Eqs. 9-11.
-constexpr int kGhostLanes = 8;
+constexpr int kGhostLanes = 8, kGhostThreads = 64;
 
 __device__ inline double quad_sum(double v) {
   v += __shfl_xor_sync(0xffffffffu, v, 4, kGhostLanes);
@@ -112,37 +112,33 @@ __device__ __forceinline__ void ho_ghost_body(const GhostParams& P, const double
         if (k < nr) acc[sd][k] = fma(coef[(size_t)k * P.rcap + a], ua, acc[sd][k]);
     }
   }
-#pragma unroll
-  for (int sd = 0; sd < 2; ++sd)
-#pragma unroll
-    for (int k = 0; k <= W; ++k)
-      if (sd < nsides) acc[sd][k] = quad_sum(acc[sd][k]);
-  if (!live || q != 0) return;
+  // the rows' sums over the lanes, transposed (FP64 additions hold a scheduler for 64 clocks: 3 for the two
+  // rows of a 3D boundary point instead of 9, 7 instead of 24 for an order-6 interface point), then an
+  // output per lane: 61 -> 55 us at 256^3 (98 k points), 24 -> 20.6 at 96^3, 16.5 -> 14.4 at 64^3 (interface)
+  __shared__ double sums[kGhostThreads / kGhostLanes][2 * (W + 1)];
+  double* sum = sums[threadIdx.x / kGhostLanes];
+  if (P.interface_) lane_sums<kGhostLanes, 2 * (W + 1)>(&acc[0][0], q, sum);
+  else lane_sums<kGhostLanes, W>(&acc[0][0], q, sum);
+  __syncwarp();
+  if (!live) return;
   if (!P.interface_) {
     const double data = P.with_data ? P.g[c] : 0.0;
-#pragma unroll
-    for (int k = 0; k < W; ++k) P.G[(size_t)c * W + k] = acc[0][k] + P.fit_cdat[(size_t)c * rows + k] * data;
+    if (q < W) P.G[(size_t)c * W + q] = sum[q] + P.fit_cdat[(size_t)c * rows + q] * data;
     return;
   }
+  if (q >= 2 * W) return;
   // Eqs. 9-11: S = b+ s+_c - b- s-_c ; ubar = -(b+ D+ - b- D-)/S
   const double *cp = P.fit_cdat + (size_t)(2 * c) * rows, *cm = P.fit_cdat + (size_t)(2 * c + 1) * rows;
   const double bp = P.beta_p, bm = P.beta_m;
   const double Sden = bp * cp[W] - bm * cm[W];
-  const double ubar = -(bp * acc[0][W] - bm * acc[1][W]) / Sden;
-  double up = ubar, um = ubar;
-  if (P.with_data) {
-    up = ubar + (P.j1[c] - bm * cm[W] * P.j0[c]) / Sden;
-    um = ubar + (P.j1[c] - bp * cp[W] * P.j0[c]) / Sden;
-  }
-#pragma unroll
-  for (int k = 0; k < W; ++k) {
-    P.G[(size_t)(2 * c) * W + k] = acc[0][k] + cp[k] * up;
-    P.G[(size_t)(2 * c + 1) * W + k] = acc[1][k] + cm[k] * um;
-  }
+  double us = -(bp * sum[W] - bm * sum[2 * W + 1]) / Sden;         // this lane's side of it
+  if (P.with_data) us += (P.j1[c] - (q < W ? bm * cm[W] : bp * cp[W]) * P.j0[c]) / Sden;
+  const int k = q < W ? q : q - W;
+  P.G[(size_t)(2 * c + (q < W ? 0 : 1)) * W + k] = sum[q < W ? k : W + 1 + k] + (q < W ? cp : cm)[k] * us;
 }
 
 template <int W>
-__global__ void __launch_bounds__(256) k_ho_ghost(GhostParams P, const double* __restrict__ u) {
+__global__ void __launch_bounds__(kGhostThreads) k_ho_ghost(GhostParams P, const double* __restrict__ u) {
   pdl_trigger();                                 // k_ho_apply's plain blocks start beside this kernel
   ho_ghost_body<W>(P, u, blockIdx.x * blockDim.x + threadIdx.x);
 }
@@ -394,9 +390,9 @@ void ho_ghost(Problem& P, const double* u, bool with_data, double* G, cudaStream
   GP.G = G;
   if (P.K_cap > 0) {
     // small blocks: a few thousand control points must still spread over all 152 SMs
-    const int grid = ceil_div((int64_t)P.K_cap * kGhostLanes, 64);
-    if (P.w == 2) IIM_LAUNCH(k_ho_ghost<2>, grid, 64, 0, s, GP, u);
-    else IIM_LAUNCH(k_ho_ghost<3>, grid, 64, 0, s, GP, u);
+    const int grid = ceil_div((int64_t)P.K_cap * kGhostLanes, kGhostThreads);
+    if (P.w == 2) IIM_LAUNCH(k_ho_ghost<2>, grid, kGhostThreads, 0, s, GP, u);
+    else IIM_LAUNCH(k_ho_ghost<3>, grid, kGhostThreads, 0, s, GP, u);
   }
 }
 
