@@ -876,10 +876,11 @@ def roofline(P, iim, torch, stream, applies_per_solve):
     (once per operator application).  Timed live with CUDA events on the problem's stream
     over repeated launches of the same kernel on the problem's own data.
 
-    Algorithmic work: fits, per fit of m rows and M monomials, Householder QR
-    2 m M^2 - 2/3 M^3 plus w+1 target rows (M^2 for R^-T, 4 m M for Q), summed over the
-    launch's fits; stencil, w(2d+1)+1 flop per unknown (16 for the 2D sixth-order
-    stencil: pair sums by |j|, then one FMA per |j| and one multiply).
+    Algorithmic work: fits, per fit of m rows and M monomials, corrected semi-normal
+    equations: 2 m K for the K moments of degree <= 2 q, M^3 / 3 for L D L^T, and per target
+    (w + 1) two solves with it (2 M^2 each) and three products with the rows (2 m M each),
+    summed over the launch's fits; stencil, w(2d+1)+1 flop per unknown (16 for the 2D
+    sixth-order stencil: pair sums by |j|, then one FMA per |j| and one multiply).
     """
     import ctypes
     lib = iim.load()
@@ -890,14 +891,16 @@ def roofline(P, iim, torch, stream, applies_per_solve):
     if lib.iim_kernel_time(P.h, 8, 20, ctypes.byref(us)) == 0:
         nfit, rows, M = iim.fit_stats(P)
         w = P.desc.order // 2
-        flops = 2.0 * M * M * rows - 2.0 / 3.0 * M ** 3 * nfit + (w + 1) * (M * M * nfit + 4.0 * M * rows)
-        out["k_fit_quad"] = {"kernel": f"k_fit_quad<{M}>", "flop": flops, "us": us.value,
+        q2 = 4 * w                                         # moments of degree <= 2 q, q = 2 w
+        K = (q2 + 1) * (q2 + 2) // 2 if P.dim == 2 else (q2 + 1) * (q2 + 2) * (q2 + 3) // 6
+        flops = 2.0 * K * rows + M ** 3 / 3.0 * nfit + (w + 1) * (4.0 * M * M * nfit + 6.0 * M * rows)
+        out["k_fit_gram"] = {"kernel": f"k_fit_gram<{M}>", "flop": flops, "us": us.value,
                              "us_per_solve": us.value}
     if lib.iim_kernel_time(P.h, 0, 50, ctypes.byref(us)) == 0:
         d, w = P.dim, P.desc.order // 2
         flops = (w * (2 * d + 1) + 1) * P.n_unknowns
-        out["k_ho_stencil"] = {"kernel": f"k_ho_stencil<{d},{w}>", "flop": flops, "us": us.value,
-                               "us_per_solve": us.value * applies_per_solve}
+        out["k_ho_apply"] = {"kernel": f"k_ho_apply<{d},{w}> (plain nodes)", "flop": flops, "us": us.value,
+                             "us_per_solve": us.value * applies_per_solve}
     if not out:
         return None
     hbm = hbm_kernels(P, iim, torch, pk)
@@ -936,7 +939,7 @@ def hbm_kernels(P, iim, torch, pk):
     rb = "16,4" if P.n >= 2048 else ("16,2" if P.n >= 512 else "8,2")
     cases = [("mg_down0", f"k_mg2d_rb<float,{rb},0> first level (down)", 18),
              ("mg_up0", f"k_mg2d_rb<float,{rb},1> first level (up)", 18),
-             ("stencil", "k_ho_stencil", 17),
+             ("stencil", "k_ho_apply (plain nodes)", 17),
              ("multidot", f"k_multidot<{j + 1}>", 8 * (j + 2)),
              ("update", f"k_update<{j + 1}>", 8 * (j + 3))]
     res = []

@@ -302,7 +302,7 @@ iim_status iim_problem_create(const iim_problem_desc* desc, const iim_options* o
       cudaEventCreateWithFlags(&P.ev_fork, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&P.ev_join, cudaEventDisableTiming) != cudaSuccess) {
     cudaGetLastError();
-    P.side = nullptr;                  // no side stream: the operator runs its kernels in sequence
+    P.side = nullptr;                  // no side stream: the set-up runs its parts in sequence
   }
   // monomials of total degree <= q, graded order
   std::vector<int> mono;
