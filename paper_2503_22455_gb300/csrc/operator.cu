@@ -521,8 +521,9 @@ iim_status ho_apply_noalloc(Problem& P, const double* u, double* w, bool with_da
 
 
 // ---------------------------------------------------------------------------- batched engine
-// Grouped forms of the three operator kernels.  A stencil item is four blocks of
-// the single-problem launch; ghost and correction items are one block each.
+// Three kernels, each over all slots: the sums of every node in phase, the ghosts, the corrections of
+// affected nodes, in the arithmetic of the two launches above.  A stencil item is 1024 nodes; ghost
+// and correction items are one block each.
 template <int D, int W>
 __global__ void __launch_bounds__(kEngThreads) k_eng_stencil(EngArgs A) {
   eng_for_items(A, kListStencil + (D - 2) * 2 + (W - 2), [&](int si, int item) {
@@ -673,10 +674,12 @@ __global__ void __launch_bounds__(64) k_boundary_values(GhostParams P, const dou
 // 1/60 for w = 3)
 struct GradCoef {
   double b[2 * kMaxW + 1];
+  double ih;                             // 1 / h
 };
 
-static GradCoef grad_coef(int w) {
+static GradCoef grad_coef(int w, double h) {
   GradCoef B;
+  B.ih = 1.0 / h;
   const double h2[2] = {2.0 / 3.0, -1.0 / 12.0};
   const double h3[3] = {3.0 / 4.0, -3.0 / 20.0, 1.0 / 60.0};
   for (int k = 0; k < 2 * kMaxW + 1; ++k) B.b[k] = 0.0;
@@ -696,31 +699,53 @@ struct GradFunctor {
   __device__ __forceinline__ double box(double v, int s) const { return s > 0 ? v : -v; }
 };
 
+// Direction k (axis k / 2, side k & 1) at affected node t: the neighbours in phase (v[j], else 0) and,
+// returned, the ghost contribution
+template <int W, class Coef>
+__device__ __forceinline__ double aff_direction(const CorrectParams& P, Coef coef, const double* __restrict__ u, int t,
+                                                int64_t i, const int* m, uint8_t ph, int k, double (&v)[W]) {
+  const int n = P.g.n, ax = k >> 1, s = k & 1 ? 1 : -1, ma = ax == 0 ? m[0] : (ax == 1 ? m[1] : m[2]);
+  const int64_t st = ax == 0 ? 1 : (ax == 1 ? (int64_t)n : (int64_t)n * n);
+#pragma unroll
+  for (int j = 1; j <= W; ++j) {
+    const int pos = ma + j * s;
+    v[j - 1] = u && pos >= 0 && pos < n && P.phase[i + j * s * st] == ph ? u[i + j * s * st] : 0.0;
+  }
+  return ho_direction(P, coef, u, t, i, m, ph, ax, k & 1);
+}
+
 // grad u by the centred first-derivative stencil b of the scheme's order, in one launch beside the
 // ghost kernel like k_ho_apply.  out is [dim][N]; zero at nodes that are not unknowns.
 template <int D, int W>
-__global__ void __launch_bounds__(256) k_grad_apply(CorrectParams P, GradCoef B, const uint8_t* __restrict__ kind,
+__global__ void __launch_bounds__(256, 6) k_grad_apply(CorrectParams P, GradCoef B, const uint8_t* __restrict__ kind,
                                                     const double* __restrict__ u, double* __restrict__ out, AffSplit S) {
   const int blk = S.index(blockIdx.x), n = P.g.n;
-  const double ih = 1.0 / P.g.h;
   if (blk < 0) {
     pdl_wait();                            // the ghost values
-    const auto A = affected<D, W, 256>(P, GradFunctor<W>{B}, u, ~blk);
     // direction 2 ax + 1 is the + side, 2 ax the - side
     if constexpr (aff_lanes<D>() == 1) {
+      const int t = ~blk * 256 + (int)threadIdx.x;
+      if (t >= min(*P.n_aff, P.n_aff_cap)) return;
+      const int64_t i = P.aff_node[t];
+      int m[3];
+      node_indices(n, D, i, m);
+      const uint8_t ph = P.phase[i];
+#pragma unroll 1
+      for (int ax = 0; ax < D; ++ax) {   // an axis at a time: few registers, so that the plain blocks' stores overlap
+        double lo[W], hi[W], acc = 0.0;
+        const double pl = aff_direction<W>(P, GradFunctor<W>{B}, u, t, i, m, ph, 2 * ax, lo);
+        const double pr = aff_direction<W>(P, GradFunctor<W>{B}, u, t, i, m, ph, 2 * ax + 1, hi);
 #pragma unroll
-      for (int ax = 0; ax < D; ++ax) {
-        double acc = 0.0;
-#pragma unroll
-        for (int j = 0; j < W; ++j) acc = fma(B.b[W + j + 1], A.v[j][2 * ax + 1] - A.v[j][2 * ax], acc);
-        if (A.live) out[(size_t)ax * P.g.N + A.i] = fma(A.part[2 * ax + 1] + A.part[2 * ax], ih, acc * ih);
+        for (int j = 0; j < W; ++j) acc = fma(B.b[W + j + 1], hi[j] - lo[j], acc);
+        out[(size_t)ax * P.g.N + i] = fma(pr + pl, B.ih, acc * B.ih);
       }
     } else {
+      const auto A = affected<D, W, 256>(P, GradFunctor<W>{B}, u, ~blk);
       double acc = 0.0;
 #pragma unroll
       for (int j = 0; j < W; ++j) acc = fma(B.b[W + j + 1], A.v[j][0] - __shfl_xor_sync(0xffffffffu, A.v[j][0], 1), acc);
       const double corr = A.part[0] + __shfl_xor_sync(0xffffffffu, A.part[0], 1);
-      if (A.live && (A.k0 & 1)) out[(size_t)(A.k0 >> 1) * P.g.N + A.i] = fma(corr, ih, acc * ih);
+      if (A.live && (A.k0 & 1)) out[(size_t)(A.k0 >> 1) * P.g.N + A.i] = fma(corr, B.ih, acc * B.ih);
     }
     return;
   }
@@ -728,15 +753,18 @@ __global__ void __launch_bounds__(256) k_grad_apply(CorrectParams P, GradCoef B,
   if (i >= P.g.N) return;
   const uint8_t kd = kind[i];
   if (kd & kKindAffected) return;
+  if (!(kd & kKindUnknown)) {
+#pragma unroll
+    for (int ax = 0; ax < D; ++ax) out[(size_t)ax * P.g.N + i] = 0.0;
+    return;
+  }
 #pragma unroll
   for (int ax = 0; ax < D; ++ax) {
     const int64_t st = ax == 0 ? 1 : (ax == 1 ? (int64_t)n : (int64_t)n * n);
     double acc = 0.0;
-    if (kd & kKindUnknown) {
 #pragma unroll
-      for (int j = 1; j <= W; ++j) acc = fma(B.b[W + j], u[i + j * st] - u[i - j * st], acc);
-    }
-    out[(size_t)ax * P.g.N + i] = acc * ih;
+    for (int j = 1; j <= W; ++j) acc = fma(B.b[W + j], u[i + j * st] - u[i - j * st], acc);
+    out[(size_t)ax * P.g.N + i] = acc * B.ih;
   }
 }
 
@@ -755,7 +783,7 @@ iim_status boundary_values(Problem& P, const double* u, double* out, cudaStream_
 }
 
 iim_status gradient(Problem& P, const double* u, double* grad, cudaStream_t s) {
-  const GradCoef B = grad_coef(P.w);
+  const GradCoef B = grad_coef(P.w, P.g.h);
   ho_ghost(P, u, true, P.G, s);                     // ghost values with the problem's data
   StencilCoef C;
   GhostParams GP;
