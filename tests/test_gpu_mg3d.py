@@ -1,6 +1,6 @@
-"""The streamed 3D multigrid kernels: one V-cycle against the oracle, and bit for bit the separate
-kernels of the batched engine, at grid sizes below, at and above the window (56 x 32 cells, one and
-several tiles, runs of two planes and more), for every condition.
+"""The 3D multigrid kernels (a launch per half sweep and transfer, u and f stored by colour): one V-cycle
+against the oracle, and bit for bit the separate kernels of the batched engine, for sizes with one to
+four levels above the tail, rows that are and are not whole warps, and every condition.
 
 Bound for FP64: the oracle's own parity bound, 1e-12 of the largest value."""
 import numpy as np
