@@ -1,0 +1,72 @@
+"""A set-up re-run with a body that needs more room than the arrays made at creation hold: the status says
+so, what the problem reports stays within its arrays, its calls stay usable, and the original body set up
+again gives what a fresh problem gives, bit for bit.
+
+The arrays hold a quarter more control points than the created body has, and 64 more.  Cases: an odd
+capacity in 2D (two fits per warp, four or eight control points per block: the last block is part full),
+both orders, 3D, and an interface (two fits per control point)."""
+import numpy as np
+import pytest
+
+import workloads as W
+from tests.gpu_helpers import dev, gpu_problem, need_gpu, set_gpu_data
+
+pytestmark = pytest.mark.gpu
+
+
+def spec_of(dim, order, n, bc, r):
+    inside = bc == W.DIRICHLET
+    return W.ProblemSpec(n=n, geometry=W.Geometry(W.CIRCLE if dim == 2 else W.SPHERE,
+                                                  ((0.013, -0.021, 0.017)[:dim] + (r,)), inside), bc=bc, order=order,
+                         box_bc=W.BOX_NONE if inside else W.BOX_DIRICHLET, beta_plus=1.5,
+                         beta_minus=0.5 if bc == W.INTERFACE else 1.0,
+                         solution=W.piecewise_polynomial(dim, 3, np.random.default_rng(n)))
+
+
+@pytest.fixture(scope="module")
+def env():
+    return need_gpu()
+
+
+def same(torch, P, Q, spec):
+    rng = np.random.default_rng(3)
+    u = dev(rng.standard_normal(P.N))
+    v = dev(rng.standard_normal(P.N) * (1 if spec.bc == W.INTERFACE else Q.phase().cpu().numpy()))
+    assert P.K == Q.K and torch.equal(P.phase(), Q.phase())
+    assert torch.equal(P.apply(u), Q.apply(u))
+    assert torch.equal(P.precondition(v), Q.precondition(v))
+    set_gpu_data(P, spec)
+    set_gpu_data(Q, spec)
+    xp, ip = P.solve()
+    xq, iq = Q.solve()
+    assert ip.converged and ip.iters == iq.iters and torch.equal(xp, xq)
+
+
+@pytest.mark.parametrize("dim,order,n,bc,r0,r1", [(2, 4, 160, W.DIRICHLET, 0.245, 0.75), (2, 6, 160, W.NEUMANN, 0.235, 0.8),
+                                                  (2, 6, 160, W.INTERFACE, 0.23, 0.8), (3, 4, 40, W.DIRICHLET, 0.3, 0.7)])
+@pytest.mark.parametrize("graph", [1, 0])
+def test_too_many_control_points(env, dim, order, n, bc, r0, r1, graph):
+    torch, iim = env
+    spec = spec_of(dim, order, n, bc, r0)
+    P = gpu_problem(iim, spec, use_graph=graph)
+    cap = P.K + P.K // 4 + 64
+    if dim == 2 and bc != W.INTERFACE:
+        assert cap % 2 == 1
+    big = gpu_problem(iim, spec_of(dim, order, n, bc, r1))
+    assert big.K > cap + 8
+    p0 = spec.geometry.params
+    P.setup(p0[:-1] + (r1,))
+    assert P.status() == iim.IIM_ERR_CAPACITY
+    assert P.refresh_sizes() <= cap
+    xc, nc = P.control_points()
+    assert xc.shape[0] == P.K
+    u = dev(np.random.default_rng(1).standard_normal(P.N))
+    P.apply(u, include_data=True)
+    P.gradient(u)
+    if bc != W.INTERFACE:
+        assert P.boundary_values(u).numel() == P.K
+    assert P.status() == iim.IIM_ERR_CAPACITY
+    P.setup(p0)
+    assert P.status() == iim.IIM_OK
+    P.refresh_sizes()
+    same(torch, P, gpu_problem(iim, spec), spec)
