@@ -45,14 +45,22 @@ __global__ void k_edge_flags(GridView g, const uint8_t* __restrict__ phase, int3
 // can count more entries than the arrays made at creation hold: the status says so, and the count is
 // cut to the capacity here, before anything reads it, so that no later kernel, copy or size query
 // goes past the arrays.
+// A level's irregular nodes (aux, cls set): one without room for its row stops being an unknown, for
+// the multigrid kernels find rows by aux in cells that cls calls irregular, and those that go by aux
+// alone read all neighbours of a cell without a row, on the grid or not.
 __global__ void k_compact(const int32_t* __restrict__ flag, const int32_t* __restrict__ id, int64_t len, int cap,
-                          int32_t* __restrict__ list, int* __restrict__ count, int* status) {
+                          int32_t* __restrict__ list, int* __restrict__ count, int32_t* __restrict__ aux,
+                          uint8_t* __restrict__ cls, int* status) {
   int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e == 0 && *count > cap) *count = cap;
   if (e >= len || !flag[e]) return;
   int c = id[e];
   if (c >= cap) {
     set_status(status, IIM_ERR_CAPACITY);
+    if (aux) {
+      aux[e] = -2;
+      cls[e] &= 4;
+    }
     return;
   }
   list[c] = (int32_t)e;
@@ -695,7 +703,7 @@ iim_status setup_geometry(Problem& P, bool size_only) {
   scan_exclusive(P.edge_flag, P.edge_id, g.N * g.dim, P.d_counts + 0, P.scan_scratch, s);
   if (size_only) return IIM_OK;
   IIM_LAUNCH(k_compact, ceil_div(g.N * g.dim, T), T, 0, s, P.edge_flag, P.edge_id, g.N * g.dim, P.K_cap, P.cr_edge,
-             P.d_counts + 0, P.d_status);
+             P.d_counts + 0, (int32_t*)nullptr, (uint8_t*)nullptr, P.d_status);
   // one warp per block: the root solves are FP64-pipe bound (16 clocks per warp instruction
   // per SM), so a few thousand control points run fastest spread one warp per SM
   IIM_LAUNCH(k_crossings, ceil_div(P.K_cap, 32), 32, 0, s, P.geom, g, P.cr_edge, P.d_counts + 0, P.K_cap, P.phase,
@@ -797,7 +805,7 @@ iim_status setup_levels(Problem& P, bool size_only) {
     scan_exclusive(L.flag, L.idx, L.g.N, P.d_counts + 2 + (int)l, P.scan_scratch, P.stream);
     if (size_only) continue;
     IIM_LAUNCH(k_compact, ceil_div(L.g.N, T), T, 0, P.stream, L.flag, L.idx, L.g.N, L.irr_cap, L.irr_node,
-               P.d_counts + 2 + (int)l, P.d_status);
+               P.d_counts + 2 + (int)l, L.aux, L.cls, P.d_status);
     fills.L[held++] = SWFill{S, L.phase, L.irr_node, P.d_counts + 2 + (int)l, L.irr_cap, L.aux, L.tab64, L.tab32};
     most = std::max(most, L.irr_cap);
     if (held == kFillLevels) fill();

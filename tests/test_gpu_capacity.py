@@ -70,3 +70,25 @@ def test_too_many_control_points(env, dim, order, n, bc, r0, r1, graph):
     assert P.status() == iim.IIM_OK
     P.refresh_sizes()
     same(torch, P, gpu_problem(iim, spec), spec)
+
+
+@pytest.mark.parametrize("dim,order,n,bc,r0,r1", [(2, 4, 160, W.DIRICHLET, 0.2, 0.75), (2, 6, 160, W.INTERFACE, 0.2, 0.8),
+                                                  (3, 4, 48, W.DIRICHLET, 0.25, 0.7), (3, 4, 48, W.INTERFACE, 0.25, 0.7)])
+@pytest.mark.parametrize("prec", [0, 1, 2])
+def test_too_many_irregular_rows(env, dim, order, n, bc, r0, r1, prec):
+    """The cells without a row take no part in the V-cycle."""
+    torch, iim = env
+    spec = spec_of(dim, order, n, bc, r0)
+    P = gpu_problem(iim, spec, mg_precision=prec)
+    p0 = spec.geometry.params
+    P.setup(p0[:-1] + (r1,))
+    assert P.status() == iim.IIM_ERR_CAPACITY
+    v = dev(np.random.default_rng(1).standard_normal(P.N))
+    z = P.precondition(v)
+    assert torch.isfinite(z).all() and torch.equal(z, P.precondition(v))
+    assert P.status() == iim.IIM_ERR_CAPACITY
+    P.setup(p0)
+    assert P.status() == iim.IIM_OK
+    P.refresh_sizes()
+    Q = gpu_problem(iim, spec, mg_precision=prec)
+    assert torch.equal(P.precondition(v), Q.precondition(v))
