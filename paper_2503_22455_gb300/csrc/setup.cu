@@ -168,7 +168,8 @@ __global__ void k_affected_fill(WalkParams P, const uint8_t* __restrict__ phase,
       int fit = -1, js = 0;
       for (int j = 1; j <= P.w; ++j) {
         int pos = m[ax] + j * s;
-        if (pos < 0 || pos >= g.n) { fit = -2; js = j; break; }
+        // off the grid: the outer box's ghosts, or, where there is no box (the status says so), none
+        if (pos < 0 || pos >= g.n) { fit = P.box_bc == IIM_BOX_DIRICHLET ? -2 : -1; js = j; break; }
         int64_t nb = i + j * s * st;
         if (phase[nb] != ph) {
           int64_t lower = s > 0 ? nb - st : nb;       // edge between offsets j-1 and j

@@ -92,3 +92,22 @@ def test_too_many_irregular_rows(env, dim, order, n, bc, r0, r1, prec):
     P.refresh_sizes()
     Q = gpu_problem(iim, spec, mg_precision=prec)
     assert torch.equal(P.precondition(v), Q.precondition(v))
+
+
+@pytest.mark.parametrize("dim,order,n,r0,r1", [(2, 4, 64, 0.8, 0.99), (2, 6, 96, 0.8, 0.99), (3, 4, 40, 0.7, 0.98)])
+def test_body_grown_into_a_box_that_is_not_there(env, dim, order, n, r0, r1):
+    """Without an outer box nothing stands behind the grid's edge: no ghost, no data."""
+    torch, iim = env
+    spec = spec_of(dim, order, n, W.DIRICHLET, r0)
+    P = gpu_problem(iim, spec)
+    p0 = spec.geometry.params
+    P.setup(p0[:-1] + (r1,))
+    assert P.status() in (iim.IIM_ERR_GEOMETRY, iim.IIM_ERR_CAPACITY)
+    P.refresh_sizes()
+    u = dev(np.zeros(P.N))
+    assert torch.isfinite(P.apply(u, include_data=True)).all()
+    assert torch.isfinite(P.gradient(u)).all()
+    P.setup(p0)
+    assert P.status() == iim.IIM_OK
+    P.refresh_sizes()
+    same(torch, P, gpu_problem(iim, spec), spec)
