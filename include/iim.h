@@ -248,7 +248,8 @@ iim_status iim_apply_noalloc(iim_problem* p, const double* u_dev, double* w_dev,
 /* b of the last iim_set_data.  Asynchronous. */
 iim_status iim_rhs(iim_problem* p, double* b_dev);
 
-/* z = one V-cycle of the Shortley-Weller multigrid applied to v / beta_sigma (Sec. 3.3). Asynchronous. */
+/* z = one V-cycle of the Shortley-Weller multigrid applied to v / beta_sigma (Sec. 3.3).  v and z may
+ * start at any double; one that is not on a 16-byte boundary costs a copy.  Asynchronous. */
 iim_status iim_precondition(iim_problem* p, const double* v_dev, double* z_dev);
 
 /* FGMRES solve of L_Omega x = b (Sec. 4.1).  x_dev: in x0, out x.  Synchronises. */

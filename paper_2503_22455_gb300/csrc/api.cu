@@ -742,7 +742,18 @@ iim_status iim_rhs(iim_problem* H, double* b) {
 
 iim_status iim_precondition(iim_problem* H, const double* v, double* z) {
   if (!H || !v || !z) return IIM_ERR_INVALID_ARG;
-  mg_precondition(H->P, v, nullptr, z, H->P.stream);
+  Problem& P = H->P;
+  // the first and last kernels of a cycle move two doubles at a time: a vector that starts between
+  // two of them (a slice of a larger buffer) goes through the problem's own
+  auto aligned = [](const double* p) { return (uintptr_t)p % sizeof(double2) == 0; };
+  const double* vi = v;
+  double* zo = aligned(z) ? z : P.tmp;
+  if (!aligned(v)) {
+    cudaMemcpyAsync(P.tmp, v, sizeof(double) * P.g.N, cudaMemcpyDeviceToDevice, P.stream);
+    vi = P.tmp;
+  }
+  mg_precondition(P, vi, nullptr, zo, P.stream);
+  if (zo != z) cudaMemcpyAsync(z, zo, sizeof(double) * P.g.N, cudaMemcpyDeviceToDevice, P.stream);
   return cuda_check("precondition");
 }
 
