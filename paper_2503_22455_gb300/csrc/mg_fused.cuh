@@ -576,6 +576,8 @@ __device__ __forceinline__ void vcycle_tail_body(const TailParams<T>& P, const d
         meet();
       }
     }
+    if (zero && its == 0)                  // no sweep (nu1 = 0) writes the u it starts from
+      for (int i = tid; i < (int)L.N; i += nt) u[i] = 0;
     __syncthreads();
   };
   // pre-smoothing of level k (the first sweep from u = 0 when zero) and the restriction
