@@ -594,7 +594,8 @@ __device__ __forceinline__ void vcycle_tail_body(const TailParams<T>& P, const d
     const T* tb = table(k);
     const T wch = DIM > 2 ? (T)0.125 : (T)0.25;
     if constexpr (F64) {
-      // a thread per node; the colour that a sweep has just solved for has none (its rounding errors)
+      // a thread per node; the colour that a sweep has just solved for has none (its rounding errors) but
+      // at nodes between walls on every side (Neumann), whose rows are zero
       const int half = (int)L.N / 2;
       for (int e = tid; e < (P.nu1 > 0 ? half : 2 * half); e += nt) {
         const int p = e < half ? e : e - half, c = sco[P.off[k] + 2 * p];
@@ -607,7 +608,10 @@ __device__ __forceinline__ void vcycle_tail_body(const TailParams<T>& P, const d
           r = f[i] - fma(row[0], u[i], tail_offdiag64<DIM>(L.n, row, u, i, m));
         }
         sr[i] = r;
-        if (P.nu1 > 0) sr[i ^ 1] = 0;
+        if (P.nu1 > 0) {
+          const int b = aux[i ^ 1];
+          sr[i ^ 1] = b != -2 && tb[b * SR] == (T)0 ? f[i ^ 1] : (T)0;
+        }
       }
       __syncthreads();
     }

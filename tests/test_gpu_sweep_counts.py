@@ -39,3 +39,20 @@ def test_cycle_matches_the_oracle(env, dim, n, bc, nu1, nu2, cycle):
         # what another problem leaves in shared memory is not read
         gpu_problem(iim, spec, mg_precision=prec).precondition(dev(1e3 * v))
         assert torch.equal(P.precondition(dev(v)), z)
+
+
+def test_nodes_between_walls_on_every_side(env):
+    """A slender tilted body whose coarse levels hold nodes with no neighbour in phase (zero Neumann rows, no
+    sweep moves them) under parents that have some: their right-hand side is a residual of either colour."""
+    torch, iim = env
+    spec = W.ProblemSpec(n=512, geometry=W.Geometry(W.ELLIPSE, (-0.1368, 0.0766, 0.3189, 0.0827, 0.297), True),
+                         bc=W.NEUMANN, order=4, box_bc=W.BOX_NONE)
+    O = OracleProblem(spec)
+    zero = [(L.n, i % L.n + i // L.n) for L in O.mg.levels[:-1] if L.n <= 32
+            for i in np.nonzero(L.unk_flat & (L.diag == 0))[0]]
+    assert any(s % 2 for _, s in zero)                 # black, on a level of the tail
+    v = np.random.default_rng(1).standard_normal(O.unk_flat.size) * O.unk_flat
+    ref = O.precondition(v)
+    for prec, tol in ((iim.MG_FP64, 1e-12), (iim.MG_FP32, 1e-5)):
+        P = gpu_problem(iim, spec, mg_precision=prec)
+        assert rel_err(P.precondition(dev(v)).cpu().numpy(), ref) < tol
