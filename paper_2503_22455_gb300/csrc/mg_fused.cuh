@@ -339,7 +339,7 @@ struct TailParams {
   int toff[kTailMaxLevels + 1];      // offsets (in T) of the levels' tables in shared memory
   const int* tcount[kTailMaxLevels]; // device counts of irregular rows per level
   int tcap[kTailMaxLevels];
-  int stage_tables;                  // 1: tables copied to shared memory
+  int stage_tables;                  // 1: tables copied to shared memory (FP64: always)
   int nu1, nu2, neumann;
   int gamma;                         // visits of the next coarser level per visit (1: V, 2: W)
   int top_visits;                    // consecutive visits of the first level (gamma when the
@@ -494,7 +494,7 @@ __device__ __forceinline__ void vcycle_tail_body(const TailParams<T>& P, const d
         sco[P.off[k] + i] = (i - r * n) | ((DIM > 2 ? r % n : r) << 10) | ((DIM > 2 ? r / n : 0) << 20);
       }
     }
-    if (P.stage_tables) {
+    if (F64 || P.stage_tables) {
       for (int k = 0; k + 1 < P.nlev; ++k) {
         const int rows = min(*P.tcount[k], P.tcap[k]);
         T* to = st + P.toff[k];
@@ -512,7 +512,7 @@ __device__ __forceinline__ void vcycle_tail_body(const TailParams<T>& P, const d
       }
     }
   }
-  auto table = [&](int k) -> const T* { return P.stage_tables ? st + P.toff[k] : P.L[k].tab; };
+  auto table = [&](int k) -> const T* { return F64 || P.stage_tables ? st + P.toff[k] : P.L[k].tab; };
   // the staging above reads set-up data only; the right-hand side below is written by the
   // kernels before this one
   pdl_trigger();

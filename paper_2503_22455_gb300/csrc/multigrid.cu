@@ -476,8 +476,14 @@ static size_t tail_start(const Problem& P) {
 size_t mg_tail_start(const Problem& P) { return tail_start(P); }
 
 // Parameters of the single-CTA tail over levels l0 .. end; *smem gets its shared
-// memory bytes.  The irregular-row tables are staged in shared memory when the
+// memory bytes.  FP32: the irregular-row tables are staged in shared memory when the
 // total stays within smem_limit (staging changes where they are read, not the result).
+// FP64 always stages them, for its sweeps take rows of a form of their own (tail_row64) and a row
+// for the regular nodes that the table does not have.  They always fit: the tail's levels hold up to
+// 4/3 kTailNodes nodes, and 5/4 as many rows with 65 more for each level.
+static_assert((2 * sizeof(double) + 2 * sizeof(int)) * (4 * kTailNodes / 3) + sizeof(double) * kTailNodes +
+                  sizeof(double) * tail_row64(3) * (5 * kTailNodes / 3 + 65 * kTailMaxLevels) <= 227 * 1024,
+              "the FP64 tail's rows must fit in shared memory");
 template <typename T>
 TailParams<T> make_tail_params(Problem& P, size_t l0, T* u_out, size_t smem_limit, size_t* smem) {
   TailParams<T> tp;
@@ -503,7 +509,7 @@ TailParams<T> make_tail_params(Problem& P, size_t l0, T* u_out, size_t smem_limi
   // u, f, aux, node coordinates; FP64: residuals of the largest level
   const size_t base = (sizeof(T) * 2 + 2 * sizeof(int)) * (size_t)off +
                       (sizeof(T) == 8 && tp.nlev > 1 ? sizeof(T) * (size_t)tp.off[1] : 0);
-  tp.stage_tables = base + sizeof(T) * (size_t)toff <= smem_limit;
+  tp.stage_tables = sizeof(T) == 8 || base + sizeof(T) * (size_t)toff <= smem_limit;
   if (!tp.stage_tables) {
     toff = 0;
     for (int k = 0; k <= tp.nlev; ++k) tp.toff[k] = 0;
