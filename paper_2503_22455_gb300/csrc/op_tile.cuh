@@ -149,6 +149,7 @@ template <int W, bool FAST, bool AFF, class Aff>
 __device__ __forceinline__ void op_tile_body(OpTile<W>& S, const GridView& g, const StencilCoef& C, bool whole,
                                              const uint8_t* __restrict__ kind, const double* __restrict__ u,
                                              double* __restrict__ w, int tile, Aff affected) {
+  static_assert(W == 2, "the sum below has a_2 = -a_1 / 16 and 60 bits for two offsets");
   using T = OpTile<W>;
   using K = TileWalk<W>;
   constexpr int TX = T::TX, TZ = T::TZ, NT = T::NT, NP = K::NP, XH = K::XH, YH = K::YH;
