@@ -476,8 +476,10 @@ __device__ void fit_cta(const FitParams& P, const int f) {
   if (tid == 0) set_status(P.status, IIM_ERR_RANK);
 }
 
-// later: a count and that many fits.  There are few or none of them, so the grid is fixed and
-// strides over the list (a CTA per possible fit cost 0.19 ms of empty CTAs at 192^3).
+// later: a count and that many fits.  Most bodies leave few or none of them, so the grid strides over
+// the list (a CTA per possible fit cost 0.19 ms of empty CTAs at 192^3); it holds as many CTAs as fit
+// the chip, for a long list: 1.6 k fits of order 4 take 0.96 ms on a CTA per SM and 0.57 so, 6.5 k of
+// order 6 10.0 and 4.6 (3D: one CTA per SM is what fits).
 __global__ void __launch_bounds__(kFitThreads) k_fit(FitParams P, const int* __restrict__ later) {
   const int count = later[0];
   for (int e = blockIdx.x; e < count; e += gridDim.x) {
@@ -778,7 +780,12 @@ iim_status setup_fits(Problem& P) {
   else
     IIM_LAUNCH(k_fit_gram<Gram24>, ceil_div(P.nfit_cap, 2), 32, 2 * sizeof(GramSmem<Gram24>), P.stream, F, P.fit_later);
   // CTA per fit for those left over (too many or too few rows for a warp, a grown region)
-  IIM_LAUNCH(k_fit, std::min(P.nfit_cap, kNumSMs), kFitThreads, smem, P.stream, F, P.fit_later);
+  int per_sm = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fit, kFitThreads, smem) != cudaSuccess || per_sm < 1) {
+    cudaGetLastError();
+    per_sm = 1;
+  }
+  IIM_LAUNCH(k_fit, std::min(P.nfit_cap, per_sm * kNumSMs), kFitThreads, smem, P.stream, F, P.fit_later);
   return IIM_OK;
 }
 
