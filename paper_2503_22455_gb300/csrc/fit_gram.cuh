@@ -18,9 +18,8 @@
 // The rank test of k_fit is on |R_kk| of the monomials around x_c.  Shifting the centre does
 // not change them (the shifted monomials are the old ones plus terms of lower degree, which
 // come earlier), so |R_kk|^2 = D_k 16^deg(k) here.  Only fits with min |R_kk| >= 1e-3 max |R_kk|
-// are taken (the test asks for 1e-8; 0.2 and 0.014 are seen); the others, those with too few or
-// too many rows for this layout and those whose control point sits on its far node are listed
-// for k_fit, which decides by QR.
+// are taken (the test asks for 1e-8; 0.2 and 0.014 are seen); the others, and those with too few or
+// too many rows for this layout, are listed for k_fit, which decides by QR.
 //
 // Layout: LANES lanes per fit (32 in 3D, 16 in 2D), rows over the lanes in three slots (a fourth
 // for fits of more than 3 LANES rows in 3D).  Sums over the rows are transposed butterflies:
@@ -353,14 +352,11 @@ __global__ void __launch_bounds__(32) k_fit_gram(FitParams P, int* __restrict__ 
   const int lo = P.cr_lo[c];
   const bool lo_sig = (P.cr_loplus[c] != 0) == sig_plus;
   const double tq = P.cr_t[c];
-  // the phase-sigma node nearest to x_c is the sigma end of the cut edge (every other node is
-  // at least h away) unless x_c sits on the far node, which k_fit's full search handles
+  // the phase-sigma node nearest to x_c is the sigma end of the cut edge, every other node being at
+  // least h away, unless x_c sits on the other end (below)
   const int st_ax = ax == 0 ? 1 : (ax == 1 ? n : n * n);
-  const int nearest = lo_sig ? lo : lo + st_ax;
-  if (active && !((lo_sig ? tq : 1.0 - tq) < 1.0 - 1e-9)) {
-    if (hl == 0) fit_append(later, f);
-    active = false;
-  }
+  int nearest = lo_sig ? lo : lo + st_ax;
+  const bool on_end = active && !((lo_sig ? tq : 1.0 - tq) < 1.0 - 1e-9);
   // ---- window coordinates
   int w0[DIM];
 #pragma unroll
@@ -369,6 +365,28 @@ __global__ void __launch_bounds__(32) k_fit_gram(FitParams P, int* __restrict__ 
     for (int i = hl; i < S::WIN; i += LN) sm.xi[k][i] = (node_x(g, w0[k] + i) - xc[k]) / g.h;
   }
   __syncwarp();
+  if (on_end) {
+    // then that end's other neighbours may be as near: the least distance, the smallest index among
+    // equals, by the expressions of k_fit.  Left to k_fit, the 1.6 k such fits of a flat-sided interface took
+    // 0.57 ms at 1024^2 (order 4), 6.5 k 4.6 ms at 4096^2 (order 6), 16 of 36 ms of set-up at 128^3.
+    const int e = lo_sig ? lo + st_ax : lo, ei[3] = {e % n, (e / n) % n, DIM == 2 ? 0 : e / n / n};
+    double bd = 1e300;
+    nearest = 0x7fffffff;
+#pragma unroll
+    for (int j = 0; j < 2 * DIM; ++j) {
+      const int pos = ei[j >> 1] + (j & 1 ? 1 : -1);
+      if (pos < 0 || pos >= n) continue;
+      const int fl = e + (j & 1 ? 1 : -1) * (j < 2 ? 1 : (j < 4 ? n : n * n));
+      if ((P.phase[fl] != 0) != sig_plus) continue;
+      double d2 = 0;
+#pragma unroll
+      for (int k = 0; k < DIM; ++k) {
+        const double rr = sm.xi[k][(k == j >> 1 ? pos : ei[k]) - w0[k]];
+        d2 = fma(rr, rr, d2);
+      }
+      better(bd, nearest, d2, fl);
+    }
+  }
   // ---- rows of X_c, in the order of the flat index
   const double an = S::q + 1.0, at = S::q / 2 + 1.0;
   int R = 0;
