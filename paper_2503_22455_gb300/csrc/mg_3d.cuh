@@ -162,37 +162,21 @@ __global__ void __launch_bounds__(256) k_smooth3d(Grid3D<T> G, T* __restrict__ u
   }
 }
 
-// two consecutive values of one colour
-template <typename T>
-struct Two {
-  T a, b;
-};
-__device__ __forceinline__ Two<float> load_two(const float* p) {
-  const float2 v = *reinterpret_cast<const float2*>(p);
-  return {v.x, v.y};
-}
-__device__ __forceinline__ Two<double> load_two(const double* p) {
-  const double2 v = *reinterpret_cast<const double2*>(p);
-  return {v.x, v.y};
-}
-__device__ __forceinline__ void store_two(float* p, float a, float b) { *reinterpret_cast<float2*>(p) = make_float2(a, b); }
-__device__ __forceinline__ void store_two(double* p, double a, double b) { *reinterpret_cast<double2*>(p) = make_double2(a, b); }
-
-// The same for levels that exceed L2 (n a multiple of 4): a thread takes two neighbouring pairs through
+// The same in FP32 for levels that exceed L2 (n a multiple of 4): a thread takes two neighbouring pairs through
 // `run` planes.  The other colour's values at its places in the next plane become the x neighbours there
 // and the z neighbours one plane on, so a plane of u crosses L2 once per run instead of three times; the
 // pairs share a vector load per neighbour row, the x neighbour between them and the index arithmetic,
 // which bounded the single pairs (99 instructions per cell, 67 % of the issue slots): 41.4 -> 30.1 us per
 // half sweep at 256^3 (17 us for its bytes), V-cycle 777 -> 689 us.
-template <typename T, bool OUT>
-__global__ void __launch_bounds__(256) k_smooth3d_run(Grid3D<T> G, T* __restrict__ u, const T* __restrict__ f,
+template <bool OUT>
+__global__ void __launch_bounds__(256) k_smooth3d_run(Grid3D<float> G, float* __restrict__ u, const float* __restrict__ f,
                                                       int f_bf16, int colour, int run, double* __restrict__ zout) {
   const int n = G.n, h = n / 2, hn = h * n, half = n * hn;
   const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = (int)(t / (unsigned)(h / 2)), k = 2 * (int)(t - (unsigned)y * (unsigned)(h / 2));
   const int z0 = blockIdx.y * run, z1 = min(n, z0 + run);
-  const T* o = u + (colour ? 0 : half);
-  T* own = u + (colour ? half : 0);
+  const float* o = u + (colour ? 0 : half);
+  float* own = u + (colour ? half : 0);
   const int fofs = colour ? half : 0;
   const bool in = y < n;
   int p = z0 * hn + y * h + k;
@@ -201,42 +185,41 @@ __global__ void __launch_bounds__(256) k_smooth3d_run(Grid3D<T> G, T* __restrict
   pdl_trigger();
   pdl_wait();
   if (!in) return;
-  const Two<T> zero = {(T)0, (T)0};
-  Two<T> om = z0 > 0 ? load_two(o + p - hn) : zero, oc = load_two(o + p);
+  auto two = [](const float* p) { return *reinterpret_cast<const float2*>(p); };
+  const float2 zero = make_float2(0.f, 0.f);
+  float2 om = z0 > 0 ? two(o + p - hn) : zero, oc = two(o + p);
   for (int z = z0; z < z1; ++z, p += hn) {
     const int e = (y + z + colour) & 1;
-    const Two<T> op = z < n - 1 ? load_two(o + p + hn) : zero;
+    const float2 op = z < n - 1 ? two(o + p + hn) : zero;
     const unsigned wn = z + 1 < z1 ? __ldg((const unsigned*)(G.cls + 2 * (p + hn))) : 0;
     const unsigned wa = (w >> (8 * e)) & 255, wb = (w >> (16 + 8 * e)) & 255;
-    T va = 0, vb = 0;
+    float va = 0, vb = 0;
     if ((wa | wb) & kClsUnknown) {
-      const T side = e ? (k + 2 < h ? o[p + 2] : (T)0) : (k > 0 ? o[p - 1] : (T)0);
-      const Two<T> ym = y > 0 ? load_two(o + p - h) : zero, yp = y < n - 1 ? load_two(o + p + h) : zero;
-      Two<T> ff;
-      if (f_bf16) ff = {load_f(f, fofs + p, f_bf16), load_f(f, fofs + p + 1, f_bf16)};
-      else ff = load_two(f + fofs + p);
-      const T a[6] = {e ? oc.a : side, e ? oc.b : oc.a, ym.a, yp.a, om.a, op.a};
-      const T b[6] = {e ? oc.b : oc.a, e ? side : oc.b, ym.b, yp.b, om.b, op.b};
+      const float side = e ? (k + 2 < h ? o[p + 2] : 0.f) : (k > 0 ? o[p - 1] : 0.f);
+      const float2 ym = y > 0 ? two(o + p - h) : zero, yp = y < n - 1 ? two(o + p + h) : zero;
+      const float2 ff = load_f2(f, fofs + p, f_bf16);
+      const float a[6] = {e ? oc.x : side, e ? oc.y : oc.x, ym.x, yp.x, om.x, op.x};
+      const float b[6] = {e ? oc.y : oc.x, e ? side : oc.y, ym.y, yp.y, om.y, op.y};
       if ((wa & wb & kClsUnknown) && !((wa | wb) & kClsIrregular)) {
-        va = mul_rn(off_residual3(ff.a, G.ih2, G.ih2, G.ih2, G.ih2, G.ih2, G.ih2, a[0], a[1], a[2], a[3], a[4], a[5]), G.inv_dreg);
-        vb = mul_rn(off_residual3(ff.b, G.ih2, G.ih2, G.ih2, G.ih2, G.ih2, G.ih2, b[0], b[1], b[2], b[3], b[4], b[5]), G.inv_dreg);
+        va = mul_rn(off_residual3(ff.x, G.ih2, G.ih2, G.ih2, G.ih2, G.ih2, G.ih2, a[0], a[1], a[2], a[3], a[4], a[5]), G.inv_dreg);
+        vb = mul_rn(off_residual3(ff.y, G.ih2, G.ih2, G.ih2, G.ih2, G.ih2, G.ih2, b[0], b[1], b[2], b[3], b[4], b[5]), G.inv_dreg);
       } else {
-        T diag, inv;
+        float diag, inv;
         if (wa & kClsUnknown) {
-          const T r = row_minus(G, 2 * k + e, y, z, (uint8_t)wa, ff.a, a, diag, inv);
+          const float r = row_minus(G, 2 * k + e, y, z, (uint8_t)wa, ff.x, a, diag, inv);
           va = mul_rn(r, inv);
         }
         if (wb & kClsUnknown) {
-          const T r = row_minus(G, 2 * k + 2 + e, y, z, (uint8_t)wb, ff.b, b, diag, inv);
+          const float r = row_minus(G, 2 * k + 2 + e, y, z, (uint8_t)wb, ff.y, b, diag, inv);
           vb = mul_rn(r, inv);
         }
       }
     }
     if (OUT) {
-      *(double2*)(zout + 2 * p) = make_double2((double)(e ? oc.a : va), (double)(e ? va : oc.a));
-      *(double2*)(zout + 2 * p + 2) = make_double2((double)(e ? oc.b : vb), (double)(e ? vb : oc.b));
+      *(double2*)(zout + 2 * p) = make_double2((double)(e ? oc.x : va), (double)(e ? va : oc.x));
+      *(double2*)(zout + 2 * p + 2) = make_double2((double)(e ? oc.y : vb), (double)(e ? vb : oc.y));
     } else {
-      store_two(own + p, va, vb);
+      *reinterpret_cast<float2*>(own + p) = make_float2(va, vb);
     }
     om = oc;
     oc = op;

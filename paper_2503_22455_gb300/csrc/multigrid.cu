@@ -746,19 +746,23 @@ static Grid3D<T> grid3d(const Level& L) {
   return G;
 }
 
-// One half sweep of a 3D level.  Levels whose u and f take more than half of L2 go through 4 planes per
-// thread, two pairs at a time (256^3: V-cycle 689 us; 8 planes 699, 16 planes 765, a pair and 16 planes
-// 777); below, a plane per thread, where the loop only adds latency (V-cycle 192^3 240 us against 249
-// with runs, 128^3 158 / 171, 96^3 101 / 128).
+// One half sweep of a 3D level.  FP32 levels from 204^3, whose u and f take more than half of L2, go
+// through 4 planes per thread, two pairs at a time; smaller ones, and FP64, a plane per thread.  V-cycle
+// in us, runs / planes: FP32 exterior 320^3 1244 / 1564, 256^3 701 / 863, 208^3 456 / 505, 192^3 336 /
+// 362 (but interior 249 / 240), 128^3 171 / 158, 96^3 128 / 101, where the loop only adds latency; FP64
+// exterior 256^3 3192 / 2924, 208^3 1977 / 1758, 176^3 1268 / 1080.  Longer runs (FP32, 256^3): 8 planes
+// 699 against 689, 16 planes 765, a pair and 16 planes 777.
 constexpr int kSmooth3dRun = 4;
 template <typename T>
 static void smooth3d(const Grid3D<T>& G, T* u, const T* f, int f_bf16, int colour, double* z, cudaStream_t s) {
   const int n = G.n;
-  if ((int64_t)n * n * n * 8 > (64 << 20) && n % 4 == 0) {
-    const dim3 grid(ceil_div((int64_t)n * (n / 4), 256), ceil_div(n, kSmooth3dRun));
-    if (z) IIM_LAUNCH_PDL((k_smooth3d_run<T, true>), grid, 256, 0, s, G, u, f, f_bf16, colour, kSmooth3dRun, z);
-    else IIM_LAUNCH_PDL((k_smooth3d_run<T, false>), grid, 256, 0, s, G, u, f, f_bf16, colour, kSmooth3dRun, z);
-    return;
+  if constexpr (sizeof(T) == 4) {
+    if ((int64_t)n * n * n * 8 > (64 << 20) && n % 4 == 0) {
+      const dim3 grid(ceil_div((int64_t)n * (n / 4), 256), ceil_div(n, kSmooth3dRun));
+      if (z) IIM_LAUNCH_PDL(k_smooth3d_run<true>, grid, 256, 0, s, G, u, f, f_bf16, colour, kSmooth3dRun, z);
+      else IIM_LAUNCH_PDL(k_smooth3d_run<false>, grid, 256, 0, s, G, u, f, f_bf16, colour, kSmooth3dRun, z);
+      return;
+    }
   }
   const dim3 grid(ceil_div((int64_t)n * (n / 2), 256), n);
   if (z) IIM_LAUNCH_PDL((k_smooth3d<T, true>), grid, 256, 0, s, G, u, f, f_bf16, colour, z);
