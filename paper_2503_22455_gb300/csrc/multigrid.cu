@@ -550,8 +550,10 @@ static void launch_tail(Problem& P, size_t l0, const double* v, const double* vs
   tp.z = z;
   // A dense inverse too large for one SM to read or (FP64) to multiply in a few us is split over a
   // cluster of eight, whose two barriers cost 1.5 us.  Tail alone / in a cluster, us, by the coarsest
-  // level's nodes (with 1024 threads): FP32 64: 17.9 / 19.4, 144: 11.8 / 12.7, 196: 13.1 / 13.0, 289: 6.9 / 5.8, 529:
-  // 11.3 / 6.6; FP64 64: 27.1 / 29.2, 100: 14.9 / 15.0, 121: 19.5 / 17.1, 289: 27.1 / 8.8, 529: 57.9 / 11.9.
+  // level's nodes: FP32 64: 14.4 / 15.5, 100: 8.9 / 9.4, 144: 10.9 / 11.0, 169: 11.1 / 11.0, 196: 12.0 /
+  // 11.4, 225: 12.1 / 11.5, 289: 8.2 / 5.1, 529: 12.8 / 6.2, 3D 125: 15.2 / 15.4, 216: 6.6 / 4.7; FP64
+  // 64: 23.7 / 23.9, 100: 13.5 / 12.1, 121: 17.9 / 13.7, 289: 27.8 / 7.7, 529: 59.3 / 12.5.  (FP32
+  // sizes between 144 and the line of 200 would gain 0.2 to 0.6 us; a batched engine's tail is always alone.)
   const bool cluster = P.coarse_n >= (sizeof(T) == 8 ? 100 : 200);
   if (cluster) smem += sizeof(T) * (size_t)P.coarse_n;
   auto run = [&](auto kernel) {
