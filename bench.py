@@ -870,6 +870,24 @@ def ncu_traffic():
     return out
 
 
+def plain_nodes(phase, n, d, w, interface):
+    """Unknowns whose neighbours up to w nodes along every axis are on the grid and of their phase (what the
+    operator's plain-node kernel computes; the affected nodes are other blocks'): their number."""
+    import torch
+    ph = phase.reshape((n,) * d).bool()
+    ok = torch.ones_like(ph) if interface else ph.clone()
+    inner = torch.zeros_like(ph)
+    inner[(slice(w, n - w),) * d] = True
+    ok &= inner
+    for ax in range(d):
+        for j in range(1, w + 1):
+            a, b = ph.narrow(ax, 0, n - j), ph.narrow(ax, j, n - j)
+            same = a == b
+            ok.narrow(ax, 0, n - j).logical_and_(same)
+            ok.narrow(ax, j, n - j).logical_and_(same)
+    return int(ok.sum())
+
+
 def roofline(P, iim, torch, stream, applies_per_solve):
     """Roofline of the dominant kernel of a solve (by device time per solve), both bound by
     the FP64 pipe: the least-squares fits (once per solve) and the high-order stencil
@@ -879,10 +897,11 @@ def roofline(P, iim, torch, stream, applies_per_solve):
     Algorithmic work: fits, per fit of m rows and M monomials, corrected semi-normal
     equations: 2 m K for the K moments of degree <= 2 q, M^3 / 3 for L D L^T, and per target
     (w + 1) two solves with it (2 M^2 each) and three products with the rows (2 m M each),
-    summed over the launch's fits; stencil, w(2d+1)+1 flop per unknown (16 for the 2D
+    summed over the launch's fits; stencil, w(2d+1)+1 flop per plain node (16 for the 2D
     sixth-order stencil: pair sums by |j|, then one FMA per |j| and one multiply).
     """
     import ctypes
+    import workloads as W
     lib = iim.load()
     pk, src = peaks()
     peak = fp64_peak_tflops(pk.get("sm_max_mhz", 2070.0))
@@ -898,7 +917,7 @@ def roofline(P, iim, torch, stream, applies_per_solve):
                              "us_per_solve": us.value}
     if lib.iim_kernel_time(P.h, 0, 50, ctypes.byref(us)) == 0:
         d, w = P.dim, P.desc.order // 2
-        flops = (w * (2 * d + 1) + 1) * P.n_unknowns
+        flops = (w * (2 * d + 1) + 1) * plain_nodes(P.phase(), P.n, d, w, P.desc.bc == W.INTERFACE)
         out["k_ho_apply"] = {"kernel": f"k_ho_apply<{d},{w}> (plain nodes)", "flop": flops, "us": us.value,
                              "us_per_solve": us.value * applies_per_solve}
     if not out:
@@ -912,7 +931,7 @@ def roofline(P, iim, torch, stream, applies_per_solve):
         return {"kernel": r["kernel"], "achieved": a, "frac": a / peak, "us_per_launch": r["us"],
                 "flop_per_launch": r["flop"], "us_per_solve": r["us_per_solve"]}
 
-    tr = ncu_traffic().get(top["kernel"])
+    tr = ncu_traffic().get(top["kernel"].split()[0])
     traffic = tr["bytes"] if tr and tr["fresh"] else None
     traffic_note = ("ncu dram__bytes_read.sum + dram__bytes_write.sum of one launch, profiles/" + tr["profile"]
                     if traffic is not None else
