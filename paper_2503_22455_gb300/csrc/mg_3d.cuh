@@ -13,8 +13,8 @@
 //     cells and for cells at a box face alone, whose weights follow from the position;
 //   - the first half sweep from u = 0 is a product and comes with the entry of f, the last one with
 //     the exit of z;
-//   - on the levels that exceed L2 a half sweep goes through several planes per thread, two pairs
-//     at a time, so that a plane crosses L2 once per run instead of three times.
+//   - on the levels that exceed L2 a half sweep in FP32 goes through several planes per thread, two
+//     pairs at a time, so that a plane crosses L2 once per run instead of three times.
 // Not kept: all four half sweeps in one kernel that streams planes through registers (1.5 ms per
 // cycle at 256^3: 500 dependent instructions per warp and plane), and the natural order of u and f
 // (0.80 ms).
